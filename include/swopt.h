@@ -73,7 +73,12 @@ typedef struct {
     double mu_per_mm;
 } swopt_switching;
 
-/* Arithmetic of the A / A^T contractions.
+/* Arithmetic of the A / A^T contractions: the values that are multiplied.  The
+ * sums are taken in FP32, by FFTs over the scan plane where the geometry allows
+ * (every precision but FP8; BF16 rounds both operands first, the split
+ * precisions keep FP32 operands), else, or when a tensor-core tiling or
+ * schedule is pinned (swopt_tc_configure, swopt_tc_schedule), by the kernels
+ * named here.
  *  SWOPT_PREC_FP32 : FP32 FMA on the CUDA cores (the accuracy reference).
  *  SWOPT_PREC_BF16 : tcgen05 tensor cores, BF16 operands, FP32 accumulation.
  *  SWOPT_PREC_BF16X3: tcgen05 tensor cores on a two-term BF16 split of both

@@ -33,7 +33,7 @@ enum {
     SC_B = 3,
     SC_C = 4,
     SC_D = 5,
-    SC_YSQ = 6,    // ||y||^2 of the measurements bound by fista_init
+    SC_YSQ = kScalYsq,  // ||y||^2 of the measurements bound by fista_init
     SC_BUDGET = 7, // refined solve: accumulated rho since the last exact gradient
     SC_COUNT = 16
 };
@@ -189,6 +189,7 @@ void release_all(swopt_handle* h)
     h->cap_stream = nullptr;
     tc_release(h);
     release_ref(h);
+    fft_release(h);
     dfree(h->Kf); dfree(h->Ka); dfree(h->fmask); dfree(h->amask); dfree(h->Sm); dfree(h->Cmf);
     dfree(h->b); dfree(h->u); dfree(h->g); dfree(h->ytil); dfree(h->red); dfree(h->scal);
     dfree(h->c); dfree(h->xi); dfree(h->zin); dfree(h->tvu); dfree(h->tvr0); dfree(h->tvr1);
@@ -268,6 +269,32 @@ swopt_status read_scalars(swopt_handle* h, cudaStream_t st)
 
 bool use_tc(const swopt_handle* h) { return h->precision != SWOPT_PREC_FP32; }
 
+// True when the spectral kernels serve the handle's precision: every one but
+// FP8, unless a tensor-core tiling or schedule is pinned (swopt_tc_configure,
+// swopt_tc_schedule), which asks for those kernels.
+bool route_fft(const swopt_handle* h)
+{
+    if (!h->fft || h->precision == SWOPT_PREC_FP8) return false;
+    if (h->precision == SWOPT_PREC_FP32) return true;
+    for (int i = 0; i < 2; ++i)
+        if (h->tc_force_mt[i] || h->tc_force_ctas[i] || h->tc_force_ra[i] ||
+            h->tc_force_split[i] || h->tc_force_nbuf[i])
+            return false;
+    return true;
+}
+
+// The tensor-core operator of the selected precision, built if the spectral
+// kernels do not serve it (synchronises; never called while capturing).
+swopt_status ensure_tc(swopt_handle* h)
+{
+    if (!use_tc(h) || h->tc) return SWOPT_OK;
+    return tc_prepare(h);
+}
+
+// SWOPT_PREC_BF16 rounds both operands of a contraction to BF16; the split
+// precisions keep (at least nearly) all of FP32, and FP32 is exact.
+bool rounds(const swopt_handle* h) { return h->precision == SWOPT_PREC_BF16; }
+
 // P then A.  out = A_OUT_U writes h->u (FP32 [Q][S][Twp]); out = A_OUT_R writes
 // the input format of apply_AT (h->u for the FP32 kernels, the padded BF16
 // residual images for the tensor-core kernels).  The result is
@@ -283,6 +310,7 @@ swopt_status no_tc_operator()
 swopt_status apply_A(swopt_handle* h, const float* c, int out, const float* ytil,
                      double* partials, int scale, cudaStream_t st)
 {
+    if (route_fft(h)) return fft_forward(h, c, ytil, scale, rounds(h), st);
     if (use_tc(h)) {
         if (!h->tc) return no_tc_operator();
         SW_TRY(tc_states(h, c, st));
@@ -296,6 +324,12 @@ swopt_status apply_A(swopt_handle* h, const float* c, int out, const float* ytil
 // apply_A(A_OUT_R).
 swopt_status apply_AT(swopt_handle* h, bool from_u, cudaStream_t st)
 {
+    if (route_fft(h)) {
+        FftImage img;
+        img.per_state = true;
+        img.out = h->g;
+        return fft_adjoint(h, h->u, false, rounds(h), img, st);
+    }
     if (use_tc(h)) {
         if (!h->tc) return no_tc_operator();
         if (from_u) SW_TRY(tc_pack_u(h, st));
@@ -307,9 +341,52 @@ swopt_status apply_AT(swopt_handle* h, bool from_u, cudaStream_t st)
 // w = H^T H v
 swopt_status normal_op(swopt_handle* h, const float* v, float* w, cudaStream_t st)
 {
+    if (route_fft(h)) {
+        FftImage img;
+        img.out = w;
+        return fft_normal(h, v, nullptr, rounds(h), FftKeep::never, img, st);
+    }
     SW_TRY(apply_A(h, v, A_OUT_R, nullptr, nullptr, 1, st));
     SW_TRY(apply_AT(h, false, st));
     return launch_pt(h, h->g, nullptr, 0.f, w, 0, st);
+}
+
+// h->g = A^T (C A P v - ytil), per state.  keep_u: h->u is written whatever the
+// measurements hold (see FftKeep).
+swopt_status state_gradient(swopt_handle* h, const float* v, const float* ytil, bool keep_u,
+                            cudaStream_t st)
+{
+    if (route_fft(h)) {
+        FftImage img;
+        img.per_state = true;
+        img.out = h->g;
+        return fft_normal(h, v, ytil, rounds(h), keep_u ? FftKeep::always : FftKeep::nonfinite, img,
+                          st);
+    }
+    SW_TRY(apply_A(h, v, A_OUT_R, ytil, nullptr, 1, st));
+    return apply_AT(h, false, st);
+}
+
+// Refined solve: G = (add ? G : 0) + P^T A^T (C A P v - ytil) and the gradient
+// step at the momentum point into h->zin (see launch_pt_refine).
+swopt_status refined_gradient(swopt_handle* h, const float* v, const float* ytil, int add,
+                              cudaStream_t st)
+{
+    const float alpha = (float)h->step;
+    if (route_fft(h)) {
+        FftImage img;
+        img.mode = 2;
+        img.add = add;
+        img.alpha = alpha;
+        img.out = h->zin;
+        img.xi = h->xi;
+        img.G = h->G;
+        return fft_normal(h, v, ytil, rounds(h), ytil ? FftKeep::nonfinite : FftKeep::never, img,
+                          st);
+    }
+    SW_TRY(apply_A(h, v, A_OUT_R, ytil, nullptr, 1, st));
+    SW_TRY(apply_AT(h, false, st));
+    return launch_pt_refine(h, h->g, h->xi, alpha, h->G, h->zin, add, st);
 }
 
 swopt_status lipschitz_impl(swopt_handle* h, const float* v0, int iters, double* L,
@@ -437,9 +514,7 @@ swopt_status validate_params(const swopt_solve_params* p)
 swopt_status exact_gradient(swopt_handle* h, cudaStream_t st)
 {
     RefScope sc(h, h->prm.refine_precision);
-    SW_TRY(apply_A(h, h->c, A_OUT_R, h->ytil, nullptr, 1, st));
-    SW_TRY(apply_AT(h, false, st));
-    return launch_pt_refine(h, h->g, h->xi, (float)h->step, h->G, h->zin, 0, st);
+    return refined_gradient(h, h->c, h->ytil, 0, st);
 }
 
 // Builds the resync precision's tensor-core operator if the refined solve
@@ -449,6 +524,7 @@ swopt_status ensure_ref(swopt_handle* h)
     const int rp = h->prm.refine_precision;
     if (h->prm.refine_every <= 0 || rp == SWOPT_PREC_FP32 || rp == h->precision) return SWOPT_OK;
     RefScope sc(h, rp);
+    if (route_fft(h)) return SWOPT_OK;
     return tc_prepare(h);
 }
 
@@ -515,8 +591,7 @@ swopt_status fista_iteration(swopt_handle* h, int kind, cudaStream_t st)
     const float alpha = (float)h->step;
     const bool refined = h->prm.refine_every > 0;
     if (!refined) {
-        SW_TRY(apply_A(h, h->xi, A_OUT_R, h->ytil, nullptr, 1, st));     // P, A, folded residual
-        SW_TRY(apply_AT(h, false, st));                                   // A^T
+        SW_TRY(state_gradient(h, h->xi, h->ytil, false, st));             // P, A, residual, A^T
         SW_TRY(launch_pt(h, h->g, h->xi, alpha, h->zin, 1, st));          // P^T, gradient step
     }
     SW_TRY(fista_prox_momentum(h, refined, st));
@@ -529,16 +604,12 @@ swopt_status fista_iteration(swopt_handle* h, int kind, cudaStream_t st)
                              h->prm.refine_budget, st));
         {
             GateScope g0(h, 0);
-            SW_TRY(apply_A(h, h->tmp, A_OUT_R, nullptr, nullptr, 1, st));
-            SW_TRY(apply_AT(h, false, st));
-            SW_TRY(launch_pt_refine(h, h->g, h->xi, alpha, h->G, h->zin, 1, st));
+            SW_TRY(refined_gradient(h, h->tmp, nullptr, 1, st));
         }
         GateScope g1(h, 1);
         return exact_gradient(h, st);
     }
-    SW_TRY(apply_A(h, h->tmp, A_OUT_R, nullptr, nullptr, 1, st));        // C A P delta
-    SW_TRY(apply_AT(h, false, st));
-    return launch_pt_refine(h, h->g, h->xi, alpha, h->G, h->zin, 1, st);
+    return refined_gradient(h, h->tmp, nullptr, 1, st);                   // C A P delta
 }
 
 // Captures one FISTA iteration into a CUDA graph on the handle's capture
@@ -781,29 +852,13 @@ swopt_status swopt_create(const swopt_geometry* geom, const double* K_host,
                     if (Kf[jd * h->Twp + tc * TCHUNK + 8 * q + i] != 0.f) msk |= (uint8_t)(1u << q);
             fm[jd * h->nTc + tc] = msk;
         }
-    std::vector<float> Ka((size_t)kk * h->Twp * h->Zp, 0.f);
-    for (int j = 0; j < g.Z; ++j)
-        for (int d = 0; d < kk; ++d)
-            for (int w = 0; w < h->Twp; ++w)
-                Ka[((size_t)d * h->Twp + w) * h->Zp + j] = Kf[((size_t)j * kk + d) * h->Twp + w];
-    std::vector<uint8_t> am((size_t)kk * h->Twp * h->nJc, 0);
-    for (size_t dw = 0; dw < (size_t)kk * h->Twp; ++dw)
-        for (int jz = 0; jz < h->nJc; ++jz) {
-            uint8_t msk = 0;
-            for (int q = 0; q < 4; ++q)
-                for (int i = 0; i < 8; ++i)
-                    if (Ka[dw * h->Zp + jz * JCHUNK + 8 * q + i] != 0.f) msk |= (uint8_t)(1u << q);
-            am[dw * h->nJc + jz] = msk;
-        }
     std::vector<float> Smf(h->Sm64.begin(), h->Sm64.end());
     std::vector<float> Cmf(h->Cm.begin(), h->Cm.end());
 
     swopt_status s = SWOPT_OK;
     auto step = [&](swopt_status v) { if (s == SWOPT_OK) s = v; };
     step(dalloc(&h->Kf, Kf.size()));
-    step(dalloc(&h->Ka, Ka.size()));
     step(dalloc(&h->fmask, fm.size()));
-    step(dalloc(&h->amask, am.size()));
     step(dalloc(&h->Sm, Smf.size()));
     step(dalloc(&h->Cmf, Cmf.size()));
     step(dalloc(&h->b, nb_of(h)));
@@ -829,9 +884,7 @@ swopt_status swopt_create(const swopt_geometry* geom, const double* K_host,
         }
     };
     up(h->Kf, Kf.data(), Kf.size() * sizeof(float));
-    up(h->Ka, Ka.data(), Ka.size() * sizeof(float));
     up(h->fmask, fm.data(), fm.size());
-    up(h->amask, am.data(), am.size());
     up(h->Sm, Smf.data(), Smf.size() * sizeof(float));
     up(h->Cmf, Cmf.data(), Cmf.size() * sizeof(float));
     if (s == SWOPT_OK) {
@@ -840,6 +893,28 @@ swopt_status swopt_create(const swopt_geometry* geom, const double* K_host,
             set_error("cudaMemset failed: %s", cudaGetErrorString(e));
             s = SWOPT_ERR_CUDA;
         }
+    }
+    if (s == SWOPT_OK) fft_prepare(h);
+    if (s == SWOPT_OK && !h->fft) {
+        // the direct FP32 adjoint's kernel copy and masks
+        std::vector<float> Ka((size_t)kk * h->Twp * h->Zp, 0.f);
+        for (int j = 0; j < g.Z; ++j)
+            for (int d = 0; d < kk; ++d)
+                for (int w = 0; w < h->Twp; ++w)
+                    Ka[((size_t)d * h->Twp + w) * h->Zp + j] = Kf[((size_t)j * kk + d) * h->Twp + w];
+        std::vector<uint8_t> am((size_t)kk * h->Twp * h->nJc, 0);
+        for (size_t dw = 0; dw < (size_t)kk * h->Twp; ++dw)
+            for (int jz = 0; jz < h->nJc; ++jz) {
+                uint8_t msk = 0;
+                for (int q = 0; q < 4; ++q)
+                    for (int i = 0; i < 8; ++i)
+                        if (Ka[dw * h->Zp + jz * JCHUNK + 8 * q + i] != 0.f) msk |= (uint8_t)(1u << q);
+                am[dw * h->nJc + jz] = msk;
+            }
+        step(dalloc(&h->Ka, Ka.size()));
+        step(dalloc(&h->amask, am.size()));
+        up(h->Ka, Ka.data(), Ka.size() * sizeof(float));
+        up(h->amask, am.data(), am.size());
     }
     if (s != SWOPT_OK) {
         release_all(h);
@@ -872,7 +947,14 @@ swopt_status swopt_set_precision(swopt_handle* h, int precision)
     if (precision != SWOPT_PREC_FP32) {
         const int prev = h->precision;
         h->precision = precision;
-        swopt_status s = tc_prepare(h);
+        // a geometry that the tensor-core kernels refuse stays refused
+        swopt_status s = tc_supported(h);
+        if (s == SWOPT_OK && rounds(h) && route_fft(h) && !fft_prepare_bf16(h)) {
+            set_error("no memory for the spectrum of the BF16 kernel");
+            s = SWOPT_ERR_OOM;
+        }
+        if (s == SWOPT_OK && route_fft(h)) tc_release(h);  // of another precision
+        else if (s == SWOPT_OK) s = tc_prepare(h);
         if (s != SWOPT_OK) {
             h->precision = prev;
             return s;
@@ -904,6 +986,11 @@ swopt_status swopt_adjoint(swopt_handle* h, const float* y_dev, float* c_dev, vo
         return SWOPT_ERR_INVALID_ARG;
     }
     cudaStream_t st = (cudaStream_t)stream;
+    if (route_fft(h)) {
+        FftImage img;
+        img.out = c_dev;
+        return fft_adjoint(h, y_dev, true, rounds(h), img, st);
+    }
     SW_TRY(launch_fold(h, y_dev, h->u, st));
     SW_TRY(apply_AT(h, true, st));
     return launch_pt(h, h->g, nullptr, 0.f, c_dev, 0, st);
@@ -1087,8 +1174,7 @@ swopt_status swopt_fista_gradient(swopt_handle* h, const float* carry_dev, float
         return SWOPT_ERR_INVALID_ARG;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    SW_TRY(apply_A(h, h->xi, A_OUT_R, h->ytil, nullptr, 1, st));
-    SW_TRY(apply_AT(h, false, st));
+    SW_TRY(state_gradient(h, h->xi, h->ytil, false, st));
     return launch_pt_carry(h, h->g, carry_dev, g_dev, st);
 }
 
@@ -1123,7 +1209,7 @@ swopt_status swopt_set_fluence(swopt_handle* h, const double* phi_host)
     switching_states(h);
     std::vector<float> Smf(h->Sm64.begin(), h->Sm64.end());
     SW_CUDA(cudaMemcpy(h->Sm, Smf.data(), Smf.size() * sizeof(float), cudaMemcpyHostToDevice));
-    return SWOPT_OK;
+    return fft_weights(h);
 }
 
 swopt_status swopt_set_state_offset(swopt_handle* h, int offset)
@@ -1139,7 +1225,7 @@ swopt_status swopt_set_state_offset(swopt_handle* h, int offset)
     switching_states(h);
     std::vector<float> Smf(h->Sm64.begin(), h->Sm64.end());
     SW_CUDA(cudaMemcpy(h->Sm, Smf.data(), Smf.size() * sizeof(float), cudaMemcpyHostToDevice));
-    return SWOPT_OK;
+    return fft_weights(h);
 }
 
 swopt_status swopt_refine_stats(swopt_handle* h, int64_t* iterations, int64_t* resyncs,
@@ -1435,8 +1521,7 @@ swopt_status swopt_param_grad(swopt_handle* h, const float* c_dev, const float* 
     float* yt = nullptr;
     SW_TRY(dalloc(&yt, nu_of(h)));
     swopt_status s = launch_fold(h, y_dev, yt, st);
-    if (s == SWOPT_OK) s = apply_A(h, c_dev, A_OUT_R, yt, nullptr, 1, st);
-    if (s == SWOPT_OK) s = apply_AT(h, false, st);
+    if (s == SWOPT_OK) s = state_gradient(h, c_dev, yt, true, st);
     if (s == SWOPT_OK) s = switching_gradient(h, c_dev, dkappa_host, dmu, st);
     cudaFree(yt);
     return s;
@@ -1454,8 +1539,15 @@ swopt_status swopt_param_vjp(swopt_handle* h, const float* c_dev, const float* w
     cudaStream_t st = (cudaStream_t)stream;
     // <w, dH/dtheta c> = sum_m <A^T w~_m, dS_m/dtheta c>, w~ the cotangent
     // folded over pulses of equal state (H c vanishes outside the window)
-    SW_TRY(launch_fold(h, w_dev, h->u, st));
-    SW_TRY(apply_AT(h, true, st));
+    if (route_fft(h)) {
+        FftImage img;
+        img.per_state = true;
+        img.out = h->g;
+        SW_TRY(fft_adjoint(h, w_dev, true, rounds(h), img, st));
+    } else {
+        SW_TRY(launch_fold(h, w_dev, h->u, st));
+        SW_TRY(apply_AT(h, true, st));
+    }
     return switching_gradient(h, c_dev, dkappa_host, dmu, st);
 }
 
@@ -1472,7 +1564,7 @@ swopt_status swopt_set_switching(swopt_handle* h, const swopt_switching* sw)
     switching_states(h);
     std::vector<float> Smf(h->Sm64.begin(), h->Sm64.end());
     SW_CUDA(cudaMemcpy(h->Sm, Smf.data(), Smf.size() * sizeof(float), cudaMemcpyHostToDevice));
-    return SWOPT_OK;
+    return fft_weights(h);
 }
 
 swopt_status swopt_use_graphs(swopt_handle* h, int on)
@@ -1559,6 +1651,10 @@ swopt_status swopt_issued_flops(swopt_handle* h, int kernel_id, double* flops)
         set_error("invalid arguments");
         return SWOPT_ERR_INVALID_ARG;
     }
+    if (route_fft(h)) {
+        *flops = 2.0 * fft_issued_macs(h, kernel_id);
+        return SWOPT_OK;
+    }
     if (use_tc(h)) {
         *flops = 2.0 * tc_issued_macs(h, kernel_id);
         return SWOPT_OK;
@@ -1591,10 +1687,8 @@ swopt_status swopt_tc_configure(swopt_handle* h, int kernel_id, int tiles_per_ct
     h->tc_force_ctas[kernel_id] = ctas_per_sm;
     h->tc_force_ra[kernel_id] = accumulators;
     release_ref(h);
-    if (h->tc) {
-        tc_release(h);
-        if (use_tc(h)) return tc_prepare(h);
-    }
+    tc_release(h);
+    if (use_tc(h) && !route_fft(h)) return tc_prepare(h);
     return SWOPT_OK;
 }
 
@@ -1608,6 +1702,7 @@ swopt_status swopt_tc_config(swopt_handle* h, int kernel_id, int* tiles_per_cta,
         set_error("invalid arguments");
         return SWOPT_ERR_INVALID_ARG;
     }
+    SW_TRY(ensure_tc(h));
     if (!h->tc) {
         set_error("no tensor-core precision selected");
         return SWOPT_ERR_INVALID_ARG;
@@ -1628,10 +1723,8 @@ swopt_status swopt_tc_schedule(swopt_handle* h, int kernel_id, int split, int bu
     h->tc_force_split[kernel_id] = split;
     h->tc_force_nbuf[kernel_id] = buffers;
     release_ref(h);
-    if (h->tc) {
-        tc_release(h);
-        if (use_tc(h)) return tc_prepare(h);
-    }
+    tc_release(h);
+    if (use_tc(h) && !route_fft(h)) return tc_prepare(h);
     return SWOPT_OK;
 }
 
@@ -1644,6 +1737,7 @@ swopt_status swopt_tc_schedule_info(swopt_handle* h, int kernel_id, int* split, 
         set_error("invalid arguments");
         return SWOPT_ERR_INVALID_ARG;
     }
+    SW_TRY(ensure_tc(h));
     if (!h->tc) {
         set_error("no tensor-core precision selected");
         return SWOPT_ERR_INVALID_ARG;
@@ -1779,11 +1873,17 @@ swopt_status batch_iteration_shared(swopt_batch* b, int kind, TcMulti* const* m,
 swopt_status batch_capture_shared(swopt_batch* b, int kind)
 {
     for (swopt_handle* h : b->hs)
-        if (!use_tc(h) || !h->tc) {
+        if (!use_tc(h)) {
             set_error("shared launches need tensor-core precisions");
             return SWOPT_ERR_UNSUPPORTED;
         }
     const bool refined = b->hs[0]->prm.refine_every > 0;
+    for (swopt_handle* h : b->hs) {
+        SW_TRY(ensure_tc(h));
+        if (!refined || h->prm.refine_precision == h->precision) continue;
+        RefScope r(h, h->prm.refine_precision);
+        if (use_tc(h)) SW_TRY(tc_prepare(h));
+    }
     TcMulti* m[4] = {nullptr, nullptr, nullptr, nullptr};
     const size_t keep = b->multi.size();
     auto undo = [&](swopt_status s) {

@@ -1918,23 +1918,57 @@ static swopt_status tune_dir(swopt_handle* h, bool adj, int force_mt, int force_
     return SWOPT_OK;
 }
 
-swopt_status tc_prepare(swopt_handle* h)
+// The padded sizes of the handle's geometry and precision.
+static void tc_sizes(const swopt_handle* h, TcOperator* t)
 {
-    const int terms =
-        h->precision == SWOPT_PREC_BF16X6 ? 3 : (h->precision == SWOPT_PREC_BF16X3 ? 2 : 1);
-    const bool fp8 = h->precision == SWOPT_PREC_FP8;
-    if (h->tc && h->tc->terms == terms && h->tc->fp8 == fp8) return SWOPT_OK;
-    tc_release(h);
-    TcOperator* t = new TcOperator();
-    t->terms = terms;
-    t->fp8 = fp8;
-    t->esl = fp8 ? 16 : 8;
+    t->terms = h->precision == SWOPT_PREC_BF16X6 ? 3 : (h->precision == SWOPT_PREC_BF16X3 ? 2 : 1);
+    t->fp8 = h->precision == SWOPT_PREC_FP8;
+    t->esl = t->fp8 ? 16 : 8;
     t->tilesX = (h->X + 7) / 8;
     t->tilesY = (h->Y + kTileY - 1) / kTileY;
     t->Xp = ((t->tilesX + 1) / 2) * 16 + 2 * h->r;  // room for up to 2 tiles per CTA
     t->Yp = t->tilesY * kTileY + 2 * h->r;
     t->HY = kTileY + 2 * h->r;
     t->Zp16 = ((h->Z + 2 * t->esl - 1) / (2 * t->esl)) * (2 * t->esl);
+}
+
+swopt_status tc_supported(swopt_handle* h)
+{
+    TcOperator t;
+    tc_sizes(h, &t);
+    if (h->Twp > 2 * kRows || t.Zp16 > 2 * kRows) {
+        set_error("tensor-core path supports a time window and a depth count up to 256 "
+                  "(window %d, depths %d)", h->Twp, h->Z);
+        return SWOPT_ERR_UNSUPPORTED;
+    }
+    for (int adj = 0; adj < 2; ++adj) {
+        bool fits = false;
+        for (int ra = t.terms > 1 ? 2 : 1; ra >= 1 && !fits; --ra)
+            for (const Cand& c : kCands)
+                for (int nbuf = 2; nbuf >= 1 && !fits; --nbuf) {
+                    DirHost H;
+                    fits = plan_dir(h, &t, adj != 0, c.MT, ra, nbuf, 0, 1, c.budget, &H);
+                }
+        if (!fits) {
+            set_error("no tensor-core configuration fits this geometry (k=%d, window %d, "
+                      "depths %d)", h->k, h->Twp, h->Z);
+            return SWOPT_ERR_UNSUPPORTED;
+        }
+    }
+    return SWOPT_OK;
+}
+
+swopt_status tc_prepare(swopt_handle* h)
+{
+    TcOperator* t = new TcOperator();
+    tc_sizes(h, t);
+    const int terms = t->terms;
+    const bool fp8 = t->fp8;
+    if (h->tc && h->tc->terms == terms && h->tc->fp8 == fp8) {
+        delete t;
+        return SWOPT_OK;
+    }
+    tc_release(h);
     h->tc = t;
     if (h->Twp > 2 * kRows || t->Zp16 > 2 * kRows) {
         set_error("tensor-core path supports a time window and a depth count up to 256 "

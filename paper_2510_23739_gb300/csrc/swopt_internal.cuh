@@ -44,6 +44,9 @@ void clear_error();
         if (s_ != SWOPT_OK) return s_;                                             \
     } while (0)
 
+// Slot of the FP64 device scalars that holds ||y||^2 of the bound measurements.
+constexpr int kScalYsq = 6;
+
 // Entries of the refined solve's decision log (a ring).
 constexpr int kRefineLog = 1 << 16;
 
@@ -62,6 +65,8 @@ struct DeviceBuf {
 
 // Tensor-core operator data (built lazily on first BF16 use).
 struct TcOperator;
+// Spectral operator data (built with the handle where it pays).
+struct FftOperator;
 
 struct ProfileRec {
     cudaEvent_t a, b;
@@ -174,6 +179,9 @@ struct swopt_handle {
     const int* gate = nullptr;    // while launching one branch: the gate word, else null
     int gate_want = 0;            // and the value that lets it run
 
+    // spectral path
+    swopt::FftOperator* fft = nullptr;  // null: the direct kernels serve every precision
+
     // tensor-core path
     swopt::TcOperator* tc = nullptr;      // operator of `precision`
     swopt::TcOperator* tc_ref = nullptr;  // operator of the refined solve's resync precision
@@ -281,6 +289,47 @@ void tc_config(const swopt_handle* h, int kernel, int* mt, int* ctas_per_sm, int
                int* groups, int* accumulators);
 void tc_schedule_info(const swopt_handle* h, int kernel, int* split, int* buffers, int* grid,
                       int* max_pieces);
+
+// A geometry that the tensor-core kernels do not take (UNSUPPORTED, with the
+// message of tc_prepare), without building anything.
+swopt_status tc_supported(swopt_handle* h);
+
+// Spectral contraction kernels (operator_fft.cu): A and A^T by FFT over the
+// scan plane in FP32.  fft_prepare plans and builds h->fft, or leaves it null;
+// fft_prepare_bf16 adds the spectrum of the BF16-rounded kernel (false: no
+// memory).  round: both operands rounded to BF16 as SWOPT_PREC_BF16 has them.
+void fft_prepare(swopt_handle* h);
+bool fft_prepare_bf16(swopt_handle* h);
+void fft_release(swopt_handle* h);
+// After h->Sm has changed (synchronises the device).
+swopt_status fft_weights(swopt_handle* h);
+// h->u = (scale ? Cm : 1) A P c - ytil (ytil may be null)
+swopt_status fft_forward(swopt_handle* h, const float* c, const float* ytil, int scale, bool round,
+                         cudaStream_t st);
+// What the last kernel of A^T writes: per_state, the images g [Q][Y][X][Z]
+// (mode 0); else with v = P^T A^T, mode 0 out = v, 1 out = xi - alpha v,
+// 2 as launch_pt_refine.
+struct FftImage {
+    bool per_state = false;
+    int mode = 0, add = 0;
+    float alpha = 0.f;
+    float* out = nullptr;
+    const float* xi = nullptr;
+    float* G = nullptr;
+};
+// A^T of src: h->u-like residuals [Q][Y][X][Twp], or (from_y) measurements
+// [N][Y][X][T] folded on the way.
+swopt_status fft_adjoint(swopt_handle* h, const float* src, bool from_y, bool round,
+                         const FftImage& img, cudaStream_t st);
+// A^T (C A P c - ytil) without u in between.  keep: whether h->u is written
+// too, as the direct sums need it where the result is not finite: always, or
+// only if the bound measurements (scal[kScalYsq]) hold infinities or NaNs; never
+// leaves such results NaN.
+enum class FftKeep { never, always, nonfinite };
+swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool round, FftKeep keep,
+                        const FftImage& img, cudaStream_t st);
+// Multiply-adds of the spectral product of A (0) or A^T (1)
+double fft_issued_macs(const swopt_handle* h, int kernel);
 
 // Elementwise / layout kernels (operator_simt.cu).
 swopt_status launch_states(swopt_handle* h, const float* c, float* b, cudaStream_t st);
