@@ -35,6 +35,8 @@ enum {
     SC_D = 5,
     SC_YSQ = kScalYsq,  // ||y||^2 of the measurements bound by fista_init
     SC_BUDGET = 7, // refined solve: accumulated rho since the last exact gradient
+    SC_E = 8,      // more reduction results
+    SC_F = 9,
     SC_COUNT = 16
 };
 
@@ -191,7 +193,7 @@ void release_all(swopt_handle* h)
     release_ref(h);
     fft_release(h);
     dfree(h->Kf); dfree(h->Ka); dfree(h->fmask); dfree(h->amask); dfree(h->Sm); dfree(h->Cmf);
-    dfree(h->b); dfree(h->u); dfree(h->g); dfree(h->ytil); dfree(h->red); dfree(h->scal);
+    dfree(h->b); dfree(h->u); dfree(h->g); dfree(h->ytil); dfree(h->yfold); dfree(h->red); dfree(h->scal); dfree(h->pparts);
     dfree(h->c); dfree(h->xi); dfree(h->zin); dfree(h->tvu); dfree(h->tvr0); dfree(h->tvr1);
     dfree(h->coop_bar);
     dfree(h->tmp); dfree(h->G); dfree(h->xprev); dfree(h->jw); dfree(h->ju); dfree(h->jr); dfree(h->sched); dfree(h->rlog);
@@ -713,45 +715,37 @@ swopt_status run_iteration(swopt_handle* h, cudaStream_t st)
     return SWOPT_OK;
 }
 
-// F(c) and the data fit on measurements y (FP64; slots SC_A..SC_D).
-swopt_status objective_impl(swopt_handle* h, const float* c, const float* y, double lam_l1,
-                            double lam_tv, double lam_3, double* F, double* fit, cudaStream_t st)
+// F(c) and the data fit on measurements y (FP64; slots SC_A..SC_F), in one
+// synchronisation.  bound: y are the measurements that fista_init bound, whose
+// folded sums and ||y||^2 the handle holds.
+swopt_status objective_impl(swopt_handle* h, const float* c, const float* y, bool bound,
+                            double lam_l1, double lam_tv, double lam_3, double* F, double* fit,
+                            cudaStream_t st)
 {
     SW_TRY(apply_A(h, c, A_OUT_U, nullptr, nullptr, 0, st));
-    SW_TRY(ensure_vectors(h));
-    // expand H c into the y layout chunk by chunk is avoided: the data fit is
-    // the sum over pulses of ||u[m(n)] - y[n]||^2 including the samples
-    // outside the window, computed as ||y||^2 + sum_m Cm ||u_m||^2 - 2 <u, ytil>.
-    float* yt = nullptr;
-    SW_TRY(dalloc(&yt, nu_of(h)));
-    swopt_status s = launch_fold(h, y, yt, st);
-    if (s == SWOPT_OK) s = reduce_sumsq(h, y, (size_t)h->N * h->S * h->T, SC_A, st);
-    if (s == SWOPT_OK) s = reduce_dot(h, h->u, yt, nu_of(h), SC_B, st);
-    // sum_m Cm ||u_m||^2 : one reduction per state
-    double cu = 0.0;
-    if (s == SWOPT_OK) s = read_scalars(h, st);
-    double ysq = h->scal_host[SC_A], uy = h->scal_host[SC_B];
-    for (int m = 0; m < h->Q && s == SWOPT_OK; ++m) {
-        s = reduce_sumsq(h, h->u + (size_t)m * h->S * h->Twp, (size_t)h->S * h->Twp, SC_C, st);
-        if (s == SWOPT_OK) s = read_scalars(h, st);
-        cu += h->Cm[m] * h->scal_host[SC_C];
+    // expanding H c into the y layout is avoided: the data fit is the sum over
+    // pulses of ||u[m(n)] - y[n]||^2 including the samples outside the window,
+    // computed as ||y||^2 + sum_m Cm ||u_m||^2 - 2 <u, ytil>.
+    const float* yt = h->ytil;
+    if (!bound) {
+        if (!h->yfold) SW_TRY(dalloc(&h->yfold, nu_of(h)));
+        yt = h->yfold;
+        SW_TRY(launch_fold(h, y, h->yfold, st));
+        SW_TRY(reduce_sumsq(h, y, (size_t)h->N * h->S * h->T, SC_A, st));
     }
-    if (s == SWOPT_OK) s = reduce_abs(h, c, nc_of(h), SC_C, st);
-    if (s == SWOPT_OK) s = reduce_tv(h, c, SC_D, st);
-    if (s == SWOPT_OK) s = read_scalars(h, st);
-    const double l1 = h->scal_host[SC_C], tvc = h->scal_host[SC_D];
-    double tvs = 0.0;  // sum_n TV((S c)^n) = sum_m Cm TV(S_m c)
-    if (s == SWOPT_OK && lam_3 != 0.0) {
-        s = launch_states(h, c, h->b, st);
-        if (s == SWOPT_OK) s = reduce_tv_states(h, h->b, SC_D, st);
-        if (s == SWOPT_OK) s = read_scalars(h, st);
-        tvs = h->scal_host[SC_D];
+    SW_TRY(reduce_dot(h, h->u, yt, nu_of(h), SC_B, st));
+    SW_TRY(reduce_states(h, h->u, SC_E, st));
+    SW_TRY(reduce_abs(h, c, nc_of(h), SC_C, st));
+    SW_TRY(reduce_tv(h, c, SC_D, st));
+    if (lam_3 != 0.0) {  // sum_n TV((S c)^n) = sum_m Cm TV(S_m c)
+        SW_TRY(launch_states(h, c, h->b, st));
+        SW_TRY(reduce_tv_states(h, h->b, SC_F, st));
     }
-    cudaFree(yt);
-    SW_TRY(s);
-    const double df = 0.5 * (ysq + cu - 2.0 * uy);
+    SW_TRY(read_scalars(h, st));
+    const double* v = h->scal_host;
+    const double df = 0.5 * (v[bound ? SC_YSQ : SC_A] + v[SC_E] - 2.0 * v[SC_B]);
     if (fit) *fit = df;
-    if (F) *F = df + lam_l1 * l1 + lam_tv * tvc + lam_3 * tvs;
+    if (F) *F = df + lam_l1 * v[SC_C] + lam_tv * v[SC_D] + (lam_3 != 0.0 ? lam_3 * v[SC_F] : 0.0);
     return SWOPT_OK;
 }
 
@@ -1405,8 +1399,8 @@ swopt_status swopt_solve(swopt_handle* h, const float* y_dev, float* c_dev,
         if (!tests) continue;
         double F = 0.0;
         if (prm->eps1 > 0 || prm->history_host)
-            SW_TRY(objective_impl(h, h->c, y_dev, prm->lambda_l1, prm->lambda_tv, prm->lambda_3,
-                                  &F, nullptr, st));
+            SW_TRY(objective_impl(h, h->c, y_dev, true, prm->lambda_l1, prm->lambda_tv,
+                                  prm->lambda_3, &F, nullptr, st));
         if (prm->history_host) prm->history_host[it] = F;
         bool stop = false;
         if (it >= 1 && prm->eps1 > 0 && std::fabs(F - f_prev) < prm->eps1 * std::fabs(f_prev))
@@ -1431,8 +1425,8 @@ swopt_status swopt_solve(swopt_handle* h, const float* y_dev, float* c_dev,
     if (stats) {
         stats->iters = it;
         stats->step = h->step;
-        SW_TRY(objective_impl(h, h->c, y_dev, prm->lambda_l1, prm->lambda_tv, prm->lambda_3,
-                              &stats->objective,
+        SW_TRY(objective_impl(h, h->c, y_dev, true, prm->lambda_l1, prm->lambda_tv,
+                              prm->lambda_3, &stats->objective,
                               &stats->data_fit, st));
     } else {
         SW_CUDA(cudaStreamSynchronize(st));
@@ -1503,7 +1497,7 @@ swopt_status swopt_objective(swopt_handle* h, const float* c_dev, const float* y
         set_error("invalid objective arguments");
         return SWOPT_ERR_INVALID_ARG;
     }
-    return objective_impl(h, c_dev, y_dev, lambda_l1, lambda_tv, lambda_3, F, fit,
+    return objective_impl(h, c_dev, y_dev, false, lambda_l1, lambda_tv, lambda_3, F, fit,
                           (cudaStream_t)stream);
 }
 
@@ -1518,13 +1512,10 @@ swopt_status swopt_param_grad(swopt_handle* h, const float* c_dev, const float* 
     }
     cudaStream_t st = (cudaStream_t)stream;
     // residual folded over equal states: C_m (A P c)_m - sum_{n=m mod cycle} y_n
-    float* yt = nullptr;
-    SW_TRY(dalloc(&yt, nu_of(h)));
-    swopt_status s = launch_fold(h, y_dev, yt, st);
-    if (s == SWOPT_OK) s = state_gradient(h, c_dev, yt, true, st);
-    if (s == SWOPT_OK) s = switching_gradient(h, c_dev, dkappa_host, dmu, st);
-    cudaFree(yt);
-    return s;
+    if (!h->yfold) SW_TRY(dalloc(&h->yfold, nu_of(h)));
+    SW_TRY(launch_fold(h, y_dev, h->yfold, st));
+    SW_TRY(state_gradient(h, c_dev, h->yfold, true, st));
+    return switching_gradient(h, c_dev, dkappa_host, dmu, st);
 }
 
 swopt_status swopt_param_vjp(swopt_handle* h, const float* c_dev, const float* w_dev,

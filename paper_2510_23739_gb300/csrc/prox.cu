@@ -750,29 +750,114 @@ __global__ void fista_scalars_kernel(double* scal, int mode)
 __global__ void set_scalar_kernel(double* scal, int slot, double v) { scal[slot] = v; }
 
 // ---- deterministic FP64 reductions (pass 1: fixed grid; pass 2: one block) ----
-__global__ void red_sumsq_kernel(const float* __restrict__ x, size_t n, double* parts)
+// Sums of products over long arrays.  FP64 arithmetic and conversions run at
+// 1/64 of the FP32 rate here: with one of each per element the sum of squares
+// of 0.42 GB took 474 us.  So a thread sums 16 products exactly enough in FP32
+// pairs first (product and its error by FMA, sum and its error by Knuth's
+// two-sum; what is dropped is below 2^-43 of the 16) and adds the pair to its
+// FP64 sum: 83 us.  Products that would leave FP32's range take FP64 throughout.
+struct PairSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x, float y)
+    {
+        const float p = x * y, e = fmaf(x, y, -p);
+        const float t = s + p, z = t - s;
+        c += ((s - (t - z)) + (p - z)) + e;
+        s = t;
+    }
+};
+
+constexpr float kPairLow = 9.094947e-13f;  // 2^-40
+constexpr float kPairHigh = 1.15292150e18f;  // 2^60
+
+// True if the pair arithmetic holds for products of values up to amax.
+__device__ __forceinline__ bool pair_range(float amax)
+{
+    return amax == 0.f || (amax >= kPairLow && amax <= kPairHigh);
+}
+
+template <int N>
+__device__ __forceinline__ double sum_products(const float (&x)[N], const float (&y)[N])
+{
+    float ax = 0.f, ay = 0.f;
+    bool fine = true;  // fmaxf drops NaNs
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        ax = fmaxf(ax, fabsf(x[i]));
+        ay = fmaxf(ay, fabsf(y[i]));
+        fine = fine && x[i] == x[i] && y[i] == y[i];
+    }
+    if (fine && pair_range(ax) && pair_range(ay)) {
+        PairSum p;
+#pragma unroll
+        for (int i = 0; i < N; ++i) p.add(x[i], y[i]);
+        return (double)p.s + (double)p.c;
+    }
+    double s = 0.0;
+    for (int i = 0; i < N; ++i) s += (double)x[i] * (double)y[i];
+    return s;
+}
+
+// sum x y (x == y: sum of squares, read once); 16-byte loads over the first
+// n16 * 16 entries (0 if an array is not 16-byte aligned)
+__global__ void __launch_bounds__(kRedThreads) red_dot_kernel(const float* __restrict__ x,
+                                                              const float* __restrict__ y,
+                                                              size_t n, size_t n16, double* parts)
 {
     __shared__ double sh[kRedThreads / 32];
     double s = 0.0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const double v = x[i];
-        s += v * v;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    // group g of 16: float4s g % 32 + 128 (g / 32) + {0, 32, 64, 96}, so that the
+    // lanes of a warp read consecutive 16 bytes
+    for (size_t g = first; g < n16; g += stride) {
+        const size_t at = (g & 31) + (g >> 5) * 128;
+        const float4* x4 = reinterpret_cast<const float4*>(x) + at;
+        const float4* y4 = reinterpret_cast<const float4*>(y) + at;
+        float a[16], b[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = __ldg(x4 + 32 * i);
+            a[4 * i] = v.x; a[4 * i + 1] = v.y; a[4 * i + 2] = v.z; a[4 * i + 3] = v.w;
+        }
+        if (x == y) {
+            s += sum_products(a, a);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 v = __ldg(y4 + 32 * i);
+                b[4 * i] = v.x; b[4 * i + 1] = v.y; b[4 * i + 2] = v.z; b[4 * i + 3] = v.w;
+            }
+            s += sum_products(a, b);
+        }
     }
+    for (size_t i = 16 * n16 + first; i < n; i += stride) s += (double)x[i] * (double)y[i];
     s = block_sum(s, sh);
     if (threadIdx.x == 0) parts[blockIdx.x] = s;
 }
 
-__global__ void red_dot_kernel(const float* __restrict__ x, const float* __restrict__ y, size_t n,
-                               double* parts)
+// parts[m gridDim.x + b] = w[m] times block b's share of the sum of squares of
+// state m's n entries (n a multiple of 32, x 16-byte aligned per state)
+__global__ void __launch_bounds__(kRedThreads) red_states_kernel(const float* __restrict__ x,
+                                                                 size_t n,
+                                                                 const float* __restrict__ w,
+                                                                 double* parts)
 {
     __shared__ double sh[kRedThreads / 32];
+    const float* xm = x + (size_t)blockIdx.y * n;
     double s = 0.0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x)
-        s += (double)x[i] * (double)y[i];
+    for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < n / 16;
+         g += (size_t)gridDim.x * blockDim.x) {
+        float a[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(xm) + 4 * g + i);
+            a[4 * i] = v.x; a[4 * i + 1] = v.y; a[4 * i + 2] = v.z; a[4 * i + 3] = v.w;
+        }
+        s += sum_products(a, a);
+    }
     s = block_sum(s, sh);
-    if (threadIdx.x == 0) parts[blockIdx.x] = s;
+    if (threadIdx.x == 0) parts[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = s * (double)w[blockIdx.y];
 }
 
 __global__ void red_abs_kernel(const float* __restrict__ x, size_t n, double* parts)
@@ -916,20 +1001,45 @@ __global__ void counter_random_kernel(float* x, size_t n, uint64_t seed)
     }
 }
 
-// W[m][p][j] = sum_s g[m][s][j] c[p][s][j] in FP64 (one thread per (m, p, j),
-// fixed order over s)
-__global__ void param_weights_kernel(const float* __restrict__ g, const float* __restrict__ c,
-                                     double* __restrict__ W, int Q, int P, int S, int Z)
+// W[m][p][j] = sum_s g[m][s][j] c[p][s][j]: block (chunk, m, species in fours)
+// sums its run of positions, lanes along j; parts[chunk][m][p][j] are then
+// added in chunk order.  Products are summed as in red_dot_kernel, 16 positions
+// at a time.  One thread per (m, p, j) over all positions, as it was, left all
+// but a few warps of the chip idle: 600 us at 48 x 48 x 117, now 12 us.
+__global__ void __launch_bounds__(128) param_partial_kernel(const float* __restrict__ g,
+                                                            const float* __restrict__ c,
+                                                            double* __restrict__ parts, int Q,
+                                                            int P, int S, int Z, int run)
 {
-    const int n = Q * P * Z;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int j = i % Z;
-        const int p = (i / Z) % P;
-        const int m = i / (Z * P);
+    const int m = blockIdx.y, p0 = 4 * blockIdx.z;
+    const int s0 = blockIdx.x * run, s1 = min(S, s0 + run);
+    for (int j = threadIdx.x; j < Z; j += blockDim.x) {
         const float* gm = g + (size_t)m * S * Z + j;
-        const float* cp = c + (size_t)p * S * Z + j;
+        for (int p = p0; p < min(P, p0 + 4); ++p) {
+            const float* cp = c + (size_t)p * S * Z + j;
+            double w = 0.0;
+            int q = s0;
+            for (; q + 16 <= s1; q += 16) {
+                float x[16], y[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    x[i] = __ldg(gm + (size_t)(q + i) * Z);
+                    y[i] = __ldg(cp + (size_t)(q + i) * Z);
+                }
+                w += sum_products(x, y);
+            }
+            for (; q < s1; ++q) w += (double)gm[(size_t)q * Z] * (double)cp[(size_t)q * Z];
+            parts[(((size_t)blockIdx.x * Q + m) * P + p) * Z + j] = w;
+        }
+    }
+}
+
+__global__ void param_final_kernel(const double* __restrict__ parts, double* __restrict__ W, int n,
+                                   int chunks)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double s = 0.0;
-        for (int q = 0; q < S; ++q) s += (double)gm[(size_t)q * Z] * (double)cp[(size_t)q * Z];
+        for (int k = 0; k < chunks; ++k) s += parts[(size_t)k * n + i];
         W[i] = s;
     }
 }
@@ -1124,17 +1234,26 @@ static swopt_status finish_reduction(swopt_handle* h, int count, int slot, cudaS
 
 swopt_status reduce_sumsq(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st)
 {
-    red_sumsq_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(x, n, h->red);
-    SW_LAUNCHED(h);
-    return finish_reduction(h, kRedBlocks, slot, st);
+    return reduce_dot(h, x, x, n, slot, st);
 }
 
 swopt_status reduce_dot(swopt_handle* h, const float* x, const float* y, size_t n, int slot,
                         cudaStream_t st)
 {
-    red_dot_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(x, y, n, h->red);
+    // whole warps of 16-element groups (512 entries)
+    const bool vec = (((uintptr_t)x | (uintptr_t)y) & 15u) == 0;
+    red_dot_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(x, y, n, vec ? n / 512 * 32 : 0, h->red);
     SW_LAUNCHED(h);
     return finish_reduction(h, kRedBlocks, slot, st);
+}
+
+swopt_status reduce_states(swopt_handle* h, const float* u, int slot, cudaStream_t st)
+{
+    const int bx = std::max(1, kRedBlocks / h->Q);
+    red_states_kernel<<<dim3(bx, h->Q), kRedThreads, 0, st>>>(u, (size_t)h->S * h->Twp, h->Cmf,
+                                                              h->red);
+    SW_LAUNCHED(h);
+    return finish_reduction(h, bx * h->Q, slot, st);
 }
 
 swopt_status reduce_abs(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st)
@@ -1200,8 +1319,14 @@ swopt_status param_weights(swopt_handle* h, const float* g, const float* c, int 
                            cudaStream_t st)
 {
     const int n = h->Q * h->P * h->Z;
-    param_weights_kernel<<<(n + 127) / 128, 128, 0, st>>>(g, c, h->red + slot0, h->Q, h->P, h->S,
-                                                          h->Z);
+    // runs of whole 16s, enough of them for about eight blocks per SM
+    const int run = std::max(16, (h->S * h->Q / (152 * 8) + 15) / 16 * 16);
+    const int chunks = (h->S + run - 1) / run;
+    if (!h->pparts) SW_CUDA(cudaMalloc((void**)&h->pparts, sizeof(double) * (size_t)chunks * n));
+    param_partial_kernel<<<dim3(chunks, h->Q, (h->P + 3) / 4), 128, 0, st>>>(
+        g, c, h->pparts, h->Q, h->P, h->S, h->Z, run);
+    SW_LAUNCHED(h);
+    param_final_kernel<<<(n + 127) / 128, 128, 0, st>>>(h->pparts, h->red + slot0, n, chunks);
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }

@@ -142,8 +142,10 @@ struct swopt_handle {
     float* u = nullptr;           // [Q][Y][X][Twp] A output / folded residual
     float* g = nullptr;           // [Q][Y][X][Z] A^T output (before P^T)
     float* ytil = nullptr;        // [Q][Y][X][Twp] pulse-folded measurements
+    float* yfold = nullptr;       // the same of measurements given to one call (on first use)
     double* red = nullptr;        // reduction partials
     int red_cap = 0;              // capacity in doubles
+    double* pparts = nullptr;     // partial sums of param_weights (allocated on first use)
     double* scal = nullptr;       // small FP64 device scalars
     double* scal_host = nullptr;  // pinned host mirror
 
@@ -373,6 +375,8 @@ swopt_status fista_reset_scalars(swopt_handle* h, cudaStream_t st);
 swopt_status reduce_sumsq(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st);
 swopt_status reduce_dot(swopt_handle* h, const float* x, const float* y, size_t n, int slot,
                         cudaStream_t st);
+// sum_m Cm[m] ||u_m||^2 of u [Q][Y][X][Twp]
+swopt_status reduce_states(swopt_handle* h, const float* u, int slot, cudaStream_t st);
 swopt_status reduce_abs(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st);
 swopt_status reduce_tv(swopt_handle* h, const float* x, int slot, cudaStream_t st);
 // sum_m Cm[m] TV(b_m) of the Q state images b [Q][Y][X][Z] (= sum_n TV((S c)^n))
