@@ -1085,6 +1085,8 @@ swopt_status coop_prepare(swopt_handle* h)
         SW_CUDA(cudaMalloc((void**)&h->coop_bar, 8 * sizeof(unsigned)));
         SW_CUDA(cudaMemset(h->coop_bar, 0, 8 * sizeof(unsigned)));
     }
+    SW_TRY(march_prepare(h));
+    if (h->march.TY > 0) return SWOPT_OK;
     if (h->tile_ty == 0) {
         // shared-memory tile: the fewest ghosted columns per SM with every tile
         // co-resident; else (tile_ty = -1) the global-memory kernel
@@ -1163,6 +1165,8 @@ static swopt_status launch_coop(swopt_handle* h, FgpCoop& a, cudaStream_t st)
 swopt_status prox_tv_coop(swopt_handle* h, const float* z, float tau, int iters,
                           int inner_momentum, float* out, cudaStream_t st)
 {
+    if (h->march.TY > 0)
+        return march_launch(h, MarchCall{z, tau, iters, inner_momentum, 0, out, nullptr, 0.f}, st);
     FgpCoop a{};
     a.z = z; a.u = h->tvu; a.r0 = h->tvr0; a.r1 = h->tvr1;
     a.v = vol_of(h); a.tau = tau; a.iters = iters; a.inner_momentum = inner_momentum;
@@ -1173,6 +1177,9 @@ swopt_status prox_tv_coop(swopt_handle* h, const float* z, float tau, int iters,
 swopt_status fista_prox_finish(swopt_handle* h, const float* z, float tau, int iters,
                                int inner_momentum, float theta, float* delta, cudaStream_t st)
 {
+    if (h->march.TY > 0)
+        return march_launch(h, MarchCall{z, tau, iters, inner_momentum, 1, nullptr, delta, theta},
+                            st);
     FgpCoop a{};
     a.z = z; a.u = h->tvu; a.r0 = h->tvr0; a.r1 = h->tvr1;
     a.v = vol_of(h); a.tau = tau; a.iters = iters; a.inner_momentum = inner_momentum;
@@ -1196,6 +1203,8 @@ int coop_error_word(swopt_handle* h)
     if (cudaMemcpy(w, h->coop_bar, sizeof(w), cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
     if (w[2] == 0) return 0;
     cudaMemset(h->coop_bar, 0, sizeof(w));
+    // blocks that gave up may have stopped at different counts
+    if (h->march.flags) cudaMemset(h->march.flags, 0, sizeof(unsigned) * h->march.blocks);
     return 1;
 }
 

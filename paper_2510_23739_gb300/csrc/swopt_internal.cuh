@@ -103,6 +103,13 @@ struct IterGraph {
     std::vector<GraphProbe> probes;
 };
 
+// On-chip TV prox (prox_march.cu): tile of TY x TX columns per block, SP
+// species at a time (TY 0: not chosen, -1: the volume does not fit).
+struct MarchPlan {
+    int TY = 0, TX = 0, SP = 0, blocks = 0;
+    unsigned* flags = nullptr;  // [blocks] iterations finished, over all launches
+};
+
 }  // namespace swopt
 
 struct swopt_handle {
@@ -163,6 +170,7 @@ struct swopt_handle {
     float* tvr1 = nullptr;        // [3][..] (pong)
     unsigned* coop_bar = nullptr; // grid barrier of the cooperative TV prox: count, generation, error
     int coop_blocks = 0;          // its grid size (0: not yet sized)
+    swopt::MarchPlan march;       // on-chip TV prox
     int tile_ty = 0, tile_tx = 0; // shared-memory TV prox tile (0: not chosen, -1: none fits)
     float* tmp = nullptr;         // [P][Y][X][Z] scratch (c_{k+1} - c_k in the refined solve)
     float* G = nullptr;           // [P][Y][X][Z] refined solve: gradient at c_k
@@ -366,6 +374,18 @@ swopt_status prox_tv_coop(swopt_handle* h, const float* z, float tau, int iters,
 swopt_status fista_prox_finish(swopt_handle* h, const float* z, float tau, int iters,
                                int inner_momentum, float theta, float* delta, cudaStream_t st);
 swopt_status coop_prepare(swopt_handle* h);
+// The same with the whole state on the chip, where it fits (prox_march.cu).
+struct MarchCall {
+    const float* z;
+    float tau;
+    int iters, inner_momentum;
+    int mode;      // 0: out = z - D^T u; 1: FISTA finish
+    float* out;
+    float* delta;  // mode 1, optional
+    float theta;
+};
+swopt_status march_prepare(swopt_handle* h);
+swopt_status march_launch(swopt_handle* h, const MarchCall& call, cudaStream_t st);
 // Failure-detection test hook of the cooperative kernels' grid barrier.
 swopt_status coop_debug(swopt_handle* h, unsigned phantom, unsigned poll_limit);
 // Reads and clears the cooperative kernel's barrier error word (0 = none).
