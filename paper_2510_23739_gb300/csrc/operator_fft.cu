@@ -393,10 +393,11 @@ struct XForward {
 };
 
 template <int SRC>
-__global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_forward_kernel(const XForward a)
+__global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_forward_kernel(const XForward a)
 {
     extern __shared__ float2 sm[];
     const FftShape& s = a.s;
+    grid_dependency();
     if (gated_off(s.gate, s.want)) return;
     const int lane = threadIdx.x & 31;
     const unsigned item = blockIdx.x * 32u + lane;
@@ -496,10 +497,11 @@ struct YPass {
 };
 
 template <int S>
-__global__ void __launch_bounds__(kMaxFftThreads, 2) fft_y_kernel(const YPass a)
+__global__ void __launch_bounds__(kMaxFftThreads, 3) fft_y_kernel(const YPass a)
 {
     extern __shared__ float2 sm[];
     const FftShape& s = a.s;
+    grid_dependency();
     if (gated_off(s.gate, s.want)) return;
     const unsigned item = blockIdx.x * 32u + (threadIdx.x & 31);
     const bool ok = item < a.items;
@@ -564,12 +566,65 @@ struct XInverse {
     int per_state;      // planes are states (else species, summed over the states)
 };
 
+// The values of a thread's second pass, through the shared-memory entries that
+// only it reads, around `fix`: a call on values in registers would have the
+// compiler spill them on every path.
+template <int R, class Fix>
+__device__ __forceinline__ void through_slots(float2 (&v)[R], float2* slot, Fix fix)
+{
+#pragma unroll
+    for (int i = 0; i < R; ++i) slot[i * 32] = v[i];
+    fix();
+#pragma unroll
+    for (int i = 0; i < R; ++i) v[i] = slot[i * 32];
+}
+
+// Entries i (column k1 + R1 i of the transform) of an image line that are not
+// finite, by their direct sums.
+__device__ __noinline__ void fix_image(const XInverse& a, float2* slot, int R, int k1, int R1,
+                                       int gx0, int gy, int plane, int ch)
+{
+    const FftShape& s = a.s;
+    for (int i = 0; i < R; ++i) {
+        const int o = k1 + R1 * i - s.x.pad, gx = gx0 + o;
+        if (o < 0 || o >= s.x.out || gx >= s.X) continue;
+        for (int h = 0; h < 2 && ch + h < s.Z; ++h) {
+            float* p = reinterpret_cast<float*>(slot + i * 32) + h;
+            if (isfinite(*p)) continue;
+            float acc = 0.f;
+            if (a.per_state) {
+                acc = direct_adjoint(s, a.r, a.from_y, plane, gy, gx, ch + h);
+            } else {
+                for (int m = 0; m < s.Q; ++m)
+                    acc = fmaf(s.Sm[((size_t)m * s.P + plane) * s.Z + ch + h],
+                               direct_adjoint(s, a.r, a.from_y, m, gy, gx, ch + h), acc);
+            }
+            *p = acc;
+        }
+    }
+}
+
+// The same for a line of u: columns x0 + k1 + R1 i.
+__device__ __noinline__ void fix_u(const FftShape& s, const float* c, float2* slot, int R, int k1,
+                                   int R1, int x0, int end, int gy, int m, int w)
+{
+    for (int i = 0; i < R; ++i) {
+        const int gx = x0 + k1 + R1 * i;
+        if (gx < max(0, x0 + s.x.pad) || gx >= end) continue;
+        for (int h = 0; h < 2; ++h) {
+            float* p = reinterpret_cast<float*>(slot + i * 32) + h;
+            if (!isfinite(*p)) *p = direct_forward(s, c, m, gy, gx, w + h);
+        }
+    }
+}
+
 // A^T's inverse along x: images [plane][Y][X][Z].
 template <int MODE>
-__global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_image_kernel(const XInverse a)
+__global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XInverse a)
 {
     extern __shared__ float2 sm[];
     const FftShape& s = a.s;
+    grid_dependency();
     if (gated_off(s.gate, s.want)) return;
     const unsigned item = blockIdx.x * 32u + (threadIdx.x & 31);
     const bool ok = item < a.items;
@@ -583,14 +638,6 @@ __global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_image_kernel(const XI
     const size_t YX = (size_t)s.Y * s.X;
     const float2* in = a.in + (size_t)line * s.x.L * a.C2 + q;
     const float beta = MODE == IMG_REFINE ? (float)a.scal[1] : 0.f;
-    auto direct = [&](int gx, int j) -> float {
-        if (a.per_state) return direct_adjoint(s, a.r, a.from_y, plane, gy, gx, j);
-        float acc = 0.f;
-        for (int m = 0; m < s.Q; ++m)
-            acc = fmaf(s.Sm[((size_t)m * s.P + plane) * s.Z + j],
-                       direct_adjoint(s, a.r, a.from_y, m, gy, gx, j), acc);
-        return acc;
-    };
     const bool two = ch + 1 < s.Z;
     fft_line<1>(
         s.x, sm,
@@ -608,13 +655,8 @@ __global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_image_kernel(const XI
                 return o >= 0 && o < s.x.out && gx < s.X ? gx : -1;
             };
             if (any_nonfinite(v) && kept(a.keep, a.ysq)) {
-#pragma unroll
-                for (int i = 0; i < R; ++i) {
-                    const int gx = out_x(i);
-                    if (gx < 0) continue;
-                    if (!isfinite(v[i].x)) v[i].x = direct(gx, ch);
-                    if (two && !isfinite(v[i].y)) v[i].y = direct(gx, ch + 1);
-                }
+                float2* slot = sm + k1 * R * 32 + (threadIdx.x & 31);
+                through_slots(v, slot, [&] { fix_image(a, slot, R, k1, R1, gx0, gy, plane, ch); });
             }
             const size_t base = ((size_t)plane * YX + (size_t)gy * s.X) * s.Z + ch;
             auto at = [&](int gx) { return base + (size_t)gx * s.Z; };
@@ -664,10 +706,11 @@ __global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_image_kernel(const XI
 
 // A's inverse along x: u [Q][Y][X][Twp], the scaled folded residual, zero past
 // the window.
-__global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_u_kernel(const XInverse a)
+__global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_u_kernel(const XInverse a)
 {
     extern __shared__ float2 sm[];
     const FftShape& s = a.s;
+    grid_dependency();
     if (gated_off(s.gate, s.want)) return;
     const unsigned item = blockIdx.x * 32u + (threadIdx.x & 31);
     const bool ok = item < a.items;
@@ -705,13 +748,10 @@ __global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_u_kernel(const XInver
                                           : make_float2(0.f, 0.f);
             }
             if (any_nonfinite(v)) {
-#pragma unroll
-                for (int i = 0; i < R; ++i) {
-                    const int gx = out_x(i);
-                    if (gx < 0) continue;
-                    if (!isfinite(v[i].x)) v[i].x = direct_forward(s, a.c, m, gy, gx, w);
-                    if (!isfinite(v[i].y)) v[i].y = direct_forward(s, a.c, m, gy, gx, w + 1);
-                }
+                float2* slot = sm + k1 * R * 32 + (threadIdx.x & 31);
+                through_slots(v, slot, [&] {
+                    fix_u(s, a.c, slot, R, k1, R1, gx0 - s.x.pad, min(s.X, gx0 + s.x.out), gy, m, w);
+                });
             }
 #pragma unroll
             for (int i = 0; i < R; ++i)
@@ -742,14 +782,15 @@ struct XResidual {
     const double* ysq;  // KEEP_NONFINITE: sum of squares of the measurements
 };
 
-__global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_residual_kernel(const XResidual a)
+// 112 registers: three blocks of 6 warps per SM, without spills
+__global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual a)
 {
     extern __shared__ float2 sm[];
     const FftShape& s = a.s;
+    grid_dependency();
     if (gated_off(s.gate, s.want)) return;
     const FftAxis& ax = s.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    float2* sm2 = sm + (size_t)ax.L * 32;
     const unsigned item = blockIdx.x * 32u + lane;
     const bool ok = item < a.items;
     const unsigned q = item % (unsigned)a.C2, line = item / (unsigned)a.C2;
@@ -783,13 +824,8 @@ __global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_residual_kernel(const
                                              : make_float2(0.f, 0.f);
         }
         if (ok && any_nonfinite(v)) {
-#pragma unroll
-            for (int i = 0; i < R; ++i) {
-                const int gx = k1 + R1 * i;
-                if (gx >= s.X) continue;
-                if (!isfinite(v[i].x)) v[i].x = direct_forward(s, a.c, m, row, gx, w);
-                if (!isfinite(v[i].y)) v[i].y = direct_forward(s, a.c, m, row, gx, w + 1);
-            }
+            float2* slot = sm + k1 * R * 32 + lane;
+            through_slots(v, slot, [&] { fix_u(s, a.c, slot, R, k1, R1, 0, s.X, row, m, w); });
         }
 #pragma unroll
         for (int i = 0; i < R; ++i) {
@@ -801,11 +837,13 @@ __global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_residual_kernel(const
             if (gx >= s.X) v[i] = make_float2(0.f, 0.f);
         }
         Dft<R, -1>::run(v);
-        sm2[k1 * 32 + lane] = v[0];
+        // into the entries that this thread has read
+        float2* slot = sm + k1 * R * 32 + lane;
+        slot[0] = v[0];
 #pragma unroll
         for (int i = 1; i < R; ++i) {
             const float2 t = __ldg(ax.tw + k1 * i);
-            sm2[(i * R1 + k1) * 32 + lane] = cmul(v[i], t.x, t.y);
+            slot[i * 32] = cmul(v[i], t.x, t.y);
         }
     };
 #define SW_P2(R)                                  \
@@ -814,15 +852,19 @@ __global__ void __launch_bounds__(kMaxFftThreads, 2) fft_x_residual_kernel(const
     SW_RADIX(ax.R2, SW_P2)
 #undef SW_P2
     __syncthreads();
-    auto store = [&](auto& v, int k1, int R2) {
+    // last pass of the forward transform: its first pass left entry (n2, k1) at n2 R2 + k1
+    auto last = [&](auto& v, int k1) {
         constexpr int R = sizeof(v) / sizeof(v[0]);
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[i] = sm[(i * ax.R2 + k1) * 32 + lane];
+        Dft<R, -1>::run(v);
         if (!ok) return;
 #pragma unroll
-        for (int i = 0; i < R; ++i) out[(size_t)(k1 + R2 * i) * a.C2] = v[i];
+        for (int i = 0; i < R; ++i) out[(size_t)(k1 + ax.R2 * i) * a.C2] = v[i];
     };
-#define SW_P3(R)                                  \
-    for (int k1 = warp; k1 < ax.R2; k1 += nw)     \
-        fft_pass2<R, -1>(ax.R2, k1, sm2, lane, store)
+#define SW_P3(R)                                    \
+    float2 v[R];                                    \
+    for (int k1 = warp; k1 < ax.R2; k1 += nw) last(v, k1)
     SW_RADIX(ax.R1, SW_P3)
 #undef SW_P3
 }
@@ -895,6 +937,7 @@ __global__ void __launch_bounds__(kSpecThreads, 2) spec_kernel(const Spec a)
 {
     extern __shared__ float4 sm4[];
     const FftShape& s = a.s;
+    grid_dependency();
     if (gated_off(s.gate, s.want)) return;
     constexpr int MS2 = spec_stride(MC) / 2;  // float4 per (channel, frequency)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -1549,7 +1592,7 @@ swopt_status launch_lines(swopt_handle* h, void (*kernel)(const Args), const Arg
     if (smem > 48 * 1024)
         SW_CUDA(cudaFuncSetAttribute((const void*)kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    kernel<<<(a.items + 31) / 32, 32 * fft_warps(ax), smem, st>>>(a);
+    SW_CUDA(launch_pdl(kernel, (a.items + 31) / 32, 32 * fft_warps(ax), smem, st, a));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
@@ -1577,7 +1620,7 @@ swopt_status launch_spec_mc(swopt_handle* h, const Spec& a, cudaStream_t st)
                                      (int)kSpecSmem));
     const dim3 grid((unsigned)h->fft->blocks,
                     (unsigned)(a.s.tiles * (ADJ && FUSED ? 1 : a.chunks)));
-    kernel<<<grid, 32 * warps, smem, st>>>(a);
+    SW_CUDA(launch_pdl(kernel, grid, 32 * warps, smem, st, a));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
@@ -1719,7 +1762,7 @@ swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool
                         const FftImage& img, cudaStream_t st)
 {
     FftOperator* f = h->fft;
-    const size_t smem = (size_t)f->x.L * 64 * sizeof(float2);
+    const size_t smem = (size_t)f->x.L * 32 * sizeof(float2);
     if (f->tiles > 1) {
         SW_TRY(fft_forward(h, c, ytil, 1, round, st));
         return fft_adjoint(h, h->u, false, round, img, st);
@@ -1746,8 +1789,9 @@ swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool
     prof_begin(h, 1, st, &rec);
     if (smem > 48 * 1024)
         SW_CUDA(cudaFuncSetAttribute(fft_x_residual_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
-    fft_x_residual_kernel<<<(v.items + 31) / 32, 32 * fft_warps(f->x), smem, st>>>(v);
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    SW_CUDA(launch_pdl(fft_x_residual_kernel, (v.items + 31) / 32, 32 * fft_warps(f->x), smem, st,
+                       v));
     SW_LAUNCHED(h);
     SW_TRY(adjoint_from_lines(h, s, h->u, false, v.keep, img, st));
     prof_end(h, &rec, st);

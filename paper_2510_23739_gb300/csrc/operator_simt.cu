@@ -279,6 +279,7 @@ template <int VEC>
 __global__ void expand_kernel(const float* __restrict__ u, float* __restrict__ y, int N, int S,
                               int T, int ncyc, int t0, int Twp)
 {
+    grid_dependency();
     const int lane = threadIdx.x & 31;
     const unsigned warps = gridDim.x * (blockDim.x >> 5);
     for (size_t row = blockIdx.x * (size_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -327,6 +328,7 @@ __global__ void pt_kernel(const float* __restrict__ g, const float* __restrict__
                           const float* __restrict__ xi, float alpha, float* __restrict__ out,
                           int Q, int P, int S, int Z, int mode, const float* carry)
 {
+    grid_dependency();
     const size_t SZ = (size_t)S * Z;
     const size_t n = (size_t)P * SZ;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
@@ -449,10 +451,9 @@ swopt_status launch_states(swopt_handle* h, const float* c, float* b, cudaStream
 swopt_status launch_expand(swopt_handle* h, const float* u, float* y, cudaStream_t st)
 {
     const int grid = std::min(grid_for((size_t)h->N * h->S, 8), 152 * 16);
-    if (h->T % 4 == 0 && ((uintptr_t)y & 15u) == 0)
-        expand_kernel<4><<<grid, 256, 0, st>>>(u, y, h->N, h->S, h->T, h->ncyc, h->t0, h->Twp);
-    else
-        expand_kernel<1><<<grid, 256, 0, st>>>(u, y, h->N, h->S, h->T, h->ncyc, h->t0, h->Twp);
+    const bool vec = h->T % 4 == 0 && ((uintptr_t)y & 15u) == 0;
+    SW_CUDA(launch_pdl(vec ? expand_kernel<4> : expand_kernel<1>, grid, 256, 0, st, u, y, h->N,
+                       h->S, h->T, h->ncyc, h->t0, h->Twp));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
@@ -471,8 +472,8 @@ swopt_status launch_pt(swopt_handle* h, const float* g, const float* xi, float a
                        int mode, cudaStream_t st)
 {
     const size_t n = nc_of(h);
-    pt_kernel<<<grid_for(n, 256), 256, 0, st>>>(g, h->Sm, xi, alpha, out, h->Q, h->P, h->S, h->Z,
-                                                 mode, nullptr);
+    SW_CUDA(launch_pdl(pt_kernel, std::min(grid_for(n, 256), 152 * 16), 256, 0, st, g, h->Sm, xi,
+                       alpha, out, h->Q, h->P, h->S, h->Z, mode, nullptr));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
@@ -481,8 +482,8 @@ swopt_status launch_pt_carry(swopt_handle* h, const float* g, const float* carry
                              cudaStream_t st)
 {
     const size_t n = nc_of(h);
-    pt_kernel<<<grid_for(n, 256), 256, 0, st>>>(g, h->Sm, nullptr, 0.f, out, h->Q, h->P, h->S,
-                                                 h->Z, 0, carry);
+    SW_CUDA(launch_pdl(pt_kernel, std::min(grid_for(n, 256), 152 * 16), 256, 0, st, g, h->Sm, nullptr,
+                       0.f, out, h->Q, h->P, h->S, h->Z, 0, carry));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }

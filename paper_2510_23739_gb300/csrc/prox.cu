@@ -928,6 +928,7 @@ __global__ void red_pair_kernel(const float* __restrict__ d, const float* __rest
                                 size_t n, double* parts)
 {
     __shared__ double sh[kRedThreads / 32];
+    grid_dependency();
     // a thread's few terms in FP32 (the ratio only steers the resync
     // schedule; FP64 arithmetic per element took 46 us on the large volume),
     // the block's sum in FP64
@@ -956,6 +957,7 @@ __global__ void refine_decide_kernel(const double* parts, int count, double* sca
                                      int* sched, int* rlog, int R, double budget)
 {
     __shared__ double sh[kRedThreads / 32];
+    grid_dependency();
     double sd = 0.0, sc = 0.0;
     for (int i = threadIdx.x; i < count; i += blockDim.x) {
         sd += parts[i];
@@ -1300,10 +1302,10 @@ swopt_status reduce_partials(swopt_handle* h, const double* parts, int count, in
 swopt_status refine_decide(swopt_handle* h, const float* d, const float* c, int slot, int R,
                            double budget, cudaStream_t st)
 {
-    red_pair_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(d, c, nc_of(h), h->red);
+    SW_CUDA(launch_pdl(red_pair_kernel, kRedBlocks, kRedThreads, 0, st, d, c, nc_of(h), h->red));
     SW_LAUNCHED(h);
-    refine_decide_kernel<<<1, kRedThreads, 0, st>>>(h->red, kRedBlocks, h->scal, slot, h->sched,
-                                                    h->rlog, R, budget);
+    SW_CUDA(launch_pdl(refine_decide_kernel, 1, kRedThreads, 0, st, h->red, kRedBlocks, h->scal, slot,
+                       h->sched, h->rlog, R, budget));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }

@@ -83,6 +83,34 @@ __device__ __forceinline__ bool gated_off(const int* gate, int want)
     return gate != nullptr && *(volatile const int*)gate != want;
 }
 
+// Programmatic dependent launch: the next kernel of the stream may start its
+// blocks while the last ones of this kernel run, and waits here before it
+// touches memory that an earlier kernel writes.  Every kernel launched with
+// launch_pdl calls it first (also behind a closed gate: its end then implies
+// the end of everything before it).
+__device__ __forceinline__ void grid_dependency()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t st, const A&... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // An event-record node pair of the captured FISTA iteration that brackets
 // one launch of the A (0) or A^T (1) kernel.
 struct GraphProbe {
