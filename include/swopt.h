@@ -334,8 +334,8 @@ swopt_status swopt_solve(swopt_handle* h, const float* y_dev, float* c_dev,
  * dual, output max(z - L^T u, 0).  S is the handle's switching model (pulse n
  * takes state n mod pulses_per_cycle); pulses of one state share one dual,
  * which gives the same iterates as one dual per pulse.  z_dev, x_dev: device
- * [P][Y][X][Z]; x may equal z.  Scratch ((8 P + 6 Q) volumes, Q the switching
- * states, plus P) is the handle's, allocated on the first call.  Errors:
+ * [P][Y][X][Z]; x may equal z.  Scratch ((13 P + 6 Q) volumes, Q the switching
+ * states) is the handle's, allocated on the first call.  Errors:
  * INVALID_ARG (null pointers, negative or non-finite weights, iters < 0,
  * step2 <= 0 with iters > 0), UNSUPPORTED for P > 8, OOM, CUDA.
  * Asynchronous on the stream. */

@@ -196,7 +196,7 @@ void release_all(swopt_handle* h)
     dfree(h->b); dfree(h->u); dfree(h->g); dfree(h->ytil); dfree(h->yfold); dfree(h->red); dfree(h->scal); dfree(h->pparts);
     dfree(h->c); dfree(h->xi); dfree(h->zin); dfree(h->tvu); dfree(h->tvr0); dfree(h->tvr1);
     dfree(h->coop_bar); dfree(h->march.flags);
-    dfree(h->tmp); dfree(h->G); dfree(h->xprev); dfree(h->jw); dfree(h->ju); dfree(h->jr); dfree(h->sched); dfree(h->rlog);
+    dfree(h->tmp); dfree(h->G); dfree(h->xprev); dfree(h->jw); dfree(h->ju); dfree(h->jr); dfree(h->je); dfree(h->sched); dfree(h->rlog);
     if (h->scal_host) cudaFreeHost(h->scal_host);
     h->scal_host = nullptr;
     for (auto& r : h->prof) {
@@ -573,7 +573,7 @@ swopt_status fista_prox_momentum(swopt_handle* h, bool refined, cudaStream_t st)
         // the prox input), then the momentum scalars and step
         SW_TRY(joint_prox_on(h, h->zin, h->zin, h->step, h->prm.lambda_tv, h->prm.lambda_l1,
                              h->prm.lambda_3, h->prm.inner_iters, h->jstep2,
-                             h->prm.inner_momentum, h->jw, h->ju, h->jr, st));
+                             h->prm.inner_momentum, h->jw, h->ju, h->jr, h->je, st));
         SW_TRY(fista_scalars(h, h->prm.momentum, st));
         SW_TRY(fista_finish(h, h->zin, false, 0.f, refined ? h->tmp : nullptr, st));
     } else if (tv) {

@@ -441,13 +441,13 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_forward_kernel(const 
             if (a.vec) {
 #pragma unroll
                 for (int i = 0; i < R; ++i)
-                    t[i] = inside(i) ? __ldg(reinterpret_cast<const float2*>(p + i * stride))
+                    t[i] = inside(i) ? load_produced(reinterpret_cast<const float2*>(p + i * stride))
                                      : make_float2(0.f, 0.f);
             } else {
 #pragma unroll
                 for (int i = 0; i < R; ++i) {
-                    t[i].x = inside(i) ? __ldg(p + i * stride) : 0.f;
-                    t[i].y = inside(i) && second ? __ldg(p + i * stride + 1) : 0.f;
+                    t[i].x = inside(i) ? load_produced(p + i * stride) : 0.f;
+                    t[i].y = inside(i) && second ? load_produced(p + i * stride + 1) : 0.f;
                 }
             }
 #pragma unroll
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_y_kernel(const YPass a)
 #pragma unroll
             for (int i = 0; i < R; ++i) {
                 const int n = n2 + i * R2;
-                v[i] = ok && n < rows ? __ldg(in + (size_t)n * a.width) : make_float2(0.f, 0.f);
+                v[i] = ok && n < rows ? load_produced(in + (size_t)n * a.width) : make_float2(0.f, 0.f);
             }
         },
         [&](auto& v, int k1, int R1) {
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
             constexpr int R = sizeof(v) / sizeof(v[0]);
 #pragma unroll
             for (int i = 0; i < R; ++i)
-                v[i] = ok ? __ldg(in + (size_t)(n2 + i * R2) * a.C2) : make_float2(0.f, 0.f);
+                v[i] = ok ? load_produced(in + (size_t)(n2 + i * R2) * a.C2) : make_float2(0.f, 0.f);
         },
         [&](auto& v, int k1, int R1) {
             constexpr int R = sizeof(v) / sizeof(v[0]);
@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_u_kernel(const XInver
             constexpr int R = sizeof(v) / sizeof(v[0]);
 #pragma unroll
             for (int i = 0; i < R; ++i)
-                v[i] = in_ok ? __ldg(in + (size_t)(n2 + i * R2) * a.C2) : make_float2(0.f, 0.f);
+                v[i] = in_ok ? load_produced(in + (size_t)(n2 + i * R2) * a.C2) : make_float2(0.f, 0.f);
         },
         [&](auto& v, int k1, int R1) {
             constexpr int R = sizeof(v) / sizeof(v[0]);
@@ -743,7 +743,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_u_kernel(const XInver
 #pragma unroll
             for (int i = 0; i < R; ++i) {
                 const int gx = out_x(i);
-                yt[i] = a.ytil && gx >= 0 ? __ldg(reinterpret_cast<const float2*>(
+                yt[i] = a.ytil && gx >= 0 ? load_produced(reinterpret_cast<const float2*>(
                                                 a.ytil + base + (size_t)gx * s.Twp))
                                           : make_float2(0.f, 0.f);
             }
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
         constexpr int R = sizeof(v) / sizeof(v[0]);
 #pragma unroll
         for (int i = 0; i < R; ++i)
-            v[i] = ok ? __ldg(in + (size_t)(n2 + i * R2) * a.C2) : make_float2(0.f, 0.f);
+            v[i] = ok ? load_produced(in + (size_t)(n2 + i * R2) * a.C2) : make_float2(0.f, 0.f);
     };
 #define SW_P1(R)                                  \
     for (int n2 = warp; n2 < ax.R2; n2 += nw)     \
@@ -819,7 +819,7 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
 #pragma unroll
         for (int i = 0; i < R; ++i) {
             const int gx = k1 + R1 * i;
-            yt[i] = a.ytil && ok && gx < s.X ? __ldg(reinterpret_cast<const float2*>(
+            yt[i] = a.ytil && ok && gx < s.X ? load_produced(reinterpret_cast<const float2*>(
                                                    a.ytil + base + (size_t)gx * s.Twp))
                                              : make_float2(0.f, 0.f);
         }
@@ -1004,8 +1004,8 @@ __global__ void __launch_bounds__(kSpecThreads, 2) spec_kernel(const Spec a)
                 auto unpacked = [&](int plane, bool use, float2& x0, float2& x1) {
                     const float2* p = a.in + ((size_t)plane * s.tiles + tile) * area * a.in_C2 + q;
                     const float2 none = make_float2(0.f, 0.f);
-                    const float2 z = use ? __ldg(p + at * a.in_C2) : none;
-                    const float2 zm = use ? __ldg(p + mi * a.in_C2) : none;
+                    const float2 z = use ? load_produced(p + at * a.in_C2) : none;
+                    const float2 zm = use ? load_produced(p + mi * a.in_C2) : none;
                     x0 = make_float2(z.x + zm.x, z.y - zm.y);
                     x1 = make_float2(z.y + zm.y, zm.x - z.x);
                 };

@@ -276,7 +276,7 @@ __global__ void states_kernel(const float* __restrict__ c, const float* __restri
 // floats (0.42 GB): 85 us; 289 us with 64-bit divisions per element and 4-byte
 // stores.
 template <int VEC>
-__global__ void expand_kernel(const float* __restrict__ u, float* __restrict__ y, int N, int S,
+__global__ void expand_kernel(const float* u, float* y, int N, int S,
                               int T, int ncyc, int t0, int Twp)
 {
     grid_dependency();
@@ -291,13 +291,13 @@ __global__ void expand_kernel(const float* __restrict__ u, float* __restrict__ y
             for (int t = 4 * lane; t < T; t += 128) {
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
                 const int w = t - t0;
-                if (w >= 0 && w < Twp) v = __ldg(reinterpret_cast<const float4*>(src + w));
+                if (w >= 0 && w < Twp) v = load_produced(reinterpret_cast<const float4*>(src + w));
                 __stcs(reinterpret_cast<float4*>(dst + t), v);
             }
         } else {
             for (int t = lane; t < T; t += 32) {
                 const int w = t - t0;
-                __stcs(dst + t, w >= 0 && w < Twp ? __ldg(src + w) : 0.f);
+                __stcs(dst + t, w >= 0 && w < Twp ? load_produced(src + w) : 0.f);
             }
         }
     }
@@ -324,8 +324,8 @@ __global__ void fold_kernel(const float* __restrict__ y, float* __restrict__ yti
 
 // mode 0: out[p][s][j] = sum_m Sm[m][p][j] g[m][s][j]
 // mode 1: out = xi - alpha * (that)
-__global__ void pt_kernel(const float* __restrict__ g, const float* __restrict__ Sm,
-                          const float* __restrict__ xi, float alpha, float* __restrict__ out,
+__global__ void pt_kernel(const float* g, const float* __restrict__ Sm, const float* xi, float alpha,
+                          float* out,
                           int Q, int P, int S, int Z, int mode, const float* carry)
 {
     grid_dependency();

@@ -924,7 +924,7 @@ __global__ void red_final_kernel(const double* parts, int count, double* out)
 }
 
 // parts[b] = this block's sum of d^2, parts[gridDim.x + b] = its sum of c^2
-__global__ void red_pair_kernel(const float* __restrict__ d, const float* __restrict__ c,
+__global__ void red_pair_kernel(const float* d, const float* c,
                                 size_t n, double* parts)
 {
     __shared__ double sh[kRedThreads / 32];

@@ -94,6 +94,15 @@ __device__ __forceinline__ void grid_dependency()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// A load, after grid_dependency(), of what an earlier kernel of the stream wrote:
+// an ordinary one, since the read-only path is for data that does not change
+// while the kernel is resident (its pointers carry no __restrict__ either).
+template <class T>
+__device__ __forceinline__ T load_produced(const T* p)
+{
+    return *p;
+}
+
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, const A&... args)
@@ -204,7 +213,8 @@ struct swopt_handle {
     float* G = nullptr;           // [P][Y][X][Z] refined solve: gradient at c_k
     float* jw = nullptr;          // [P][Y][X][Z] joint prox (lambda_3): projected primal point
     float* ju = nullptr;          // [(4 P + 3 Q) Y X Z] joint prox dual iterate
-    float* jr = nullptr;          // [(4 P + 3 Q) Y X Z] joint prox momentum iterate
+    float* jr = nullptr;          // [(4 P + 3 Q) Y X Z] joint prox dual iterate before it
+    float* je = nullptr;          // [4 P Y X Z] joint prox sums for L^T
     float* xprev = nullptr;       // [P][Y][X][Z] previous momentum iterate (eps2 test)
     int64_t iter = 0;             // FISTA iterations since swopt_fista_init
     int64_t resyncs = 0;          // exact gradients of the refined solve (host-scheduled)
@@ -450,7 +460,7 @@ swopt_status fista_init_impl(swopt_handle* h, const float* y, const swopt_solve_
 
 // The joint prox of R3 with its lambda_3 term (prox_joint.cu): Algorithm 2 on
 // the stacked operator with one dual per switching state, z and x may alias;
-// scratch w [P L], u and r [joint_dual_floats] (ensure_joint_buffers gives the
+// scratch w [P L], u and r [joint_dual_floats], e [4 P L] (ensure_joint_buffers gives the
 // handle's).  joint_step_bound: an upper bound of eig_max(L L^T).
 size_t joint_dual_floats(const swopt_handle* h);
 double joint_step_bound(const swopt_handle* h, double lambda_tv, double lambda_l1,
@@ -459,7 +469,7 @@ swopt_status ensure_joint_buffers(swopt_handle* h);
 swopt_status joint_prox_on(swopt_handle* h, const float* z, float* x, double alpha,
                            double lambda_tv, double lambda_l1, double lambda_b, int iters,
                            double step2, int momentum, float* w, float* u, float* r,
-                           cudaStream_t st);
+                           float* e, cudaStream_t st);
 
 // Handle-free launchers of one FGP iteration / the primal recovery on
 // caller-given buffers (prox.cu); the duals u, rin, rout have 3 components.
