@@ -392,6 +392,13 @@ swopt_status swopt_param_grad(swopt_handle* h, const float* c_dev, const float* 
 swopt_status swopt_param_vjp(swopt_handle* h, const float* c_dev, const float* w_dev,
                              double* dkappa_host, double* dmu, void* stream);
 
+/* swopt_adjoint and swopt_param_vjp of the same cotangent w_dev with one A^T
+ * between them (the backward pass of H in c, kappa and mu): gc_dev
+ * [P][Y][X][Z] = H^T w, dkappa_host and *dmu as swopt_param_vjp.
+ * Synchronises. */
+swopt_status swopt_adjoint_vjp(swopt_handle* h, const float* c_dev, const float* w_dev,
+                               float* gc_dev, double* dkappa_host, double* dmu, void* stream);
+
 /* Fluence from the diffusion equation, Eqs. (de), (bc) and
  * (diffusion-coefficient), on the GPU: cell-centred finite volumes on a
  * Y x X x Z voxel grid (lateral pitch dx_mm, depth pitch dz_mm, depth index 0

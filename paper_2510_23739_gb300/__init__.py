@@ -112,6 +112,9 @@ _SIGS = {
     "swopt_param_vjp": ([ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                          ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
                          ctypes.c_void_p], ctypes.c_int),
+    "swopt_adjoint_vjp": ([ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
+                           ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
+                           ctypes.c_void_p], ctypes.c_int),
     "swopt_set_switching": ([ctypes.c_void_p, ctypes.POINTER(_Switching)], ctypes.c_int),
     "swopt_batch_create": ([ctypes.POINTER(ctypes.c_void_p), ctypes.c_int,
                             ctypes.POINTER(ctypes.c_void_p)], ctypes.c_int),
@@ -579,6 +582,18 @@ class Operator:
                                      ctypes.byref(dmu), _stream(stream)))
         return dk, dmu.value
 
+    def adjoint_vjp(self, c, w, stream=None):
+        """(H^T w, dkappa [P], dmu): adjoint and param_vjp of one cotangent."""
+        import torch
+        gc = torch.empty(self.c_shape, device=w.device, dtype=torch.float32)
+        dk = np.zeros(self.geom.P)
+        dmu = ctypes.c_double()
+        _check(lib().swopt_adjoint_vjp(self._h, _ptr(c, self.c_shape, "c"),
+                                       _ptr(w, self.y_shape, "w"), _ptr(gc, self.c_shape, "gc"),
+                                       dk.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                                       ctypes.byref(dmu), _stream(stream)))
+        return gc, dk, dmu.value
+
     # -- instrumentation --------------------------------------------------
     def use_graphs(self, on=True):
         _check(lib().swopt_use_graphs(self._h, 1 if on else 0))
@@ -741,10 +756,15 @@ def _make_hfunction():
             if not (np.array_equal(k0, ctx.k) and m0 == ctx.m):
                 op.set_switching(kappa=ctx.k, mu=ctx.m)
             gy = gy.contiguous()
-            gc = op.adjoint(gy) if ctx.needs_input_grad[0] else None
-            gk = gm = None
-            if ctx.needs_input_grad[1] or ctx.needs_input_grad[2]:
+            gc = gk = gm = None
+            params = ctx.needs_input_grad[1] or ctx.needs_input_grad[2]
+            if ctx.needs_input_grad[0] and params:
+                gc, dk, dmu = op.adjoint_vjp(c.contiguous(), gy)
+            elif ctx.needs_input_grad[0]:
+                gc = op.adjoint(gy)
+            elif params:
                 dk, dmu = op.param_vjp(c.contiguous(), gy)
+            if params:
                 gk = torch.tensor(dk, dtype=ctx.kdtype, device=ctx.kdev)
                 gm = torch.tensor(dmu, dtype=ctx.mdtype, device=ctx.mdev)
             return gc, gk, gm, None

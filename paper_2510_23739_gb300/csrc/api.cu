@@ -148,7 +148,21 @@ void release_graph(swopt_handle* h)
     }
     for (auto& e : h->cap_events) cudaEventDestroy(e.first);
     h->cap_events.clear();
+    h->cap_valid = false;
     ++h->graph_gen;
+}
+
+// True if the handle's captured iterations were captured with its present
+// solve settings (what fista_iteration bakes into launches).
+bool same_captures(const swopt_handle* h)
+{
+    const swopt_solve_params& a = h->cap_prm;
+    const swopt_solve_params& b = h->prm;
+    return h->cap_valid && h->cap_step == h->step && h->cap_jstep2 == h->jstep2 &&
+           a.lambda_l1 == b.lambda_l1 && a.lambda_tv == b.lambda_tv && a.lambda_3 == b.lambda_3 &&
+           a.inner_iters == b.inner_iters && a.momentum == b.momentum &&
+           a.inner_momentum == b.inner_momentum && a.refine_every == b.refine_every &&
+           a.refine_precision == b.refine_precision && a.refine_budget == b.refine_budget;
 }
 
 // Within its scope the handle computes at the refined solve's resync
@@ -351,6 +365,19 @@ swopt_status normal_op(swopt_handle* h, const float* v, float* w, cudaStream_t s
     SW_TRY(apply_A(h, v, A_OUT_R, nullptr, nullptr, 1, st));
     SW_TRY(apply_AT(h, false, st));
     return launch_pt(h, h->g, nullptr, 0.f, w, 0, st);
+}
+
+// h->g = A^T of the measurements y folded over pulses of equal state, per state.
+swopt_status states_adjoint(swopt_handle* h, const float* y, cudaStream_t st)
+{
+    if (route_fft(h)) {
+        FftImage img;
+        img.per_state = true;
+        img.out = h->g;
+        return fft_adjoint(h, y, true, rounds(h), img, st);
+    }
+    SW_TRY(launch_fold(h, y, h->u, st));
+    return apply_AT(h, true, st);
 }
 
 // h->g = A^T (C A P v - ytil), per state.  keep_u: h->u is written whatever the
@@ -637,6 +664,10 @@ swopt_status build_graph(swopt_handle* h, int kind)
         set_error("graph capture failed: %s", cudaGetErrorString(e));
         return SWOPT_ERR_CUDA;
     }
+    h->cap_valid = true;
+    h->cap_prm = h->prm;
+    h->cap_step = h->step;
+    h->cap_jstep2 = h->jstep2;
     G.graph = g;
     G.kernels = h->launches - launches0;
     h->launches = launches0;
@@ -1073,7 +1104,6 @@ swopt_status fista_init_impl(swopt_handle* h, const float* y_dev, const swopt_so
 {
     SW_TRY(validate_params(prm));
     h->fista_ready = false;
-    release_graph(h);
     SW_TRY(ensure_vectors(h));
     SW_TRY(ensure_ytil(h));
     if (prm->lambda_3 > 0) {
@@ -1101,6 +1131,9 @@ swopt_status fista_init_impl(swopt_handle* h, const float* y_dev, const swopt_so
         }
         h->step = 1.0 / L;
     }
+    // captured iterations hold the settings and buffers that the handle keeps: they
+    // serve this solve too if the settings are the same
+    if (!same_captures(h)) release_graph(h);
     SW_CUDA(cudaMemsetAsync(h->c, 0, nc_of(h) * sizeof(float), st));
     SW_CUDA(cudaMemsetAsync(h->xi, 0, nc_of(h) * sizeof(float), st));
     SW_TRY(fista_reset_scalars(h, st));
@@ -1530,15 +1563,22 @@ swopt_status swopt_param_vjp(swopt_handle* h, const float* c_dev, const float* w
     cudaStream_t st = (cudaStream_t)stream;
     // <w, dH/dtheta c> = sum_m <A^T w~_m, dS_m/dtheta c>, w~ the cotangent
     // folded over pulses of equal state (H c vanishes outside the window)
-    if (route_fft(h)) {
-        FftImage img;
-        img.per_state = true;
-        img.out = h->g;
-        SW_TRY(fft_adjoint(h, w_dev, true, rounds(h), img, st));
-    } else {
-        SW_TRY(launch_fold(h, w_dev, h->u, st));
-        SW_TRY(apply_AT(h, true, st));
+    SW_TRY(states_adjoint(h, w_dev, st));
+    return switching_gradient(h, c_dev, dkappa_host, dmu, st);
+}
+
+swopt_status swopt_adjoint_vjp(swopt_handle* h, const float* c_dev, const float* w_dev,
+                               float* gc_dev, double* dkappa_host, double* dmu, void* stream)
+{
+    clear_error();
+    SW_TRY(check_handle(h));
+    if (!c_dev || !w_dev || !gc_dev || !dkappa_host || !dmu) {
+        set_error("null argument");
+        return SWOPT_ERR_INVALID_ARG;
     }
+    cudaStream_t st = (cudaStream_t)stream;
+    SW_TRY(states_adjoint(h, w_dev, st));
+    SW_TRY(launch_pt(h, h->g, nullptr, 0.f, gc_dev, 0, st));
     return switching_gradient(h, c_dev, dkappa_host, dmu, st);
 }
 

@@ -1159,17 +1159,6 @@ __global__ void __launch_bounds__(kSpecThreads, 2) spec_kernel(const Spec a)
     }
 }
 
-// S in the order the products read it: [j][m][species in fours], zero padded.
-__global__ void weights_kernel(const float* __restrict__ Sm, float* __restrict__ S4, int Q, int P,
-                               int Z, int P4)
-{
-    const int n = Z * Q * P4 * 4;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int p = i % (4 * P4), m = i / (4 * P4) % Q, j = i / (4 * P4 * Q);
-        S4[i] = p < P ? Sm[((size_t)m * P + p) * Z + j] : 0.f;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Set-up of K^ (FP64 sums of the FP32 kernel, or of its BF16 rounding), one
 // pass per lateral axis; frequencies of u[y] = sum_d b[y + d] K[d], so with
@@ -1437,14 +1426,18 @@ static bool build_spectrum(swopt_handle* h, int which)
     return ok;
 }
 
+// S in the order the products read it: [j][m][species in fours], zero padded.
 swopt_status fft_weights(swopt_handle* h)
 {
     if (!h->fft) return SWOPT_OK;
-    const int P4 = (h->P + 3) / 4, n = h->Z * h->Q * P4 * 4;
-    weights_kernel<<<std::min((n + 255) / 256, 152 * 8), 256>>>(
-        h->Sm, reinterpret_cast<float*>(h->fft->S4), h->Q, h->P, h->Z, P4);
-    SW_CUDA(cudaGetLastError());
-    SW_CUDA(cudaDeviceSynchronize());
+    const int P4 = (h->P + 3) / 4;
+    std::vector<float> w((size_t)h->Z * h->Q * P4 * 4, 0.f);
+    for (int m = 0; m < h->Q; ++m)
+        for (int p = 0; p < h->P; ++p)
+            for (int j = 0; j < h->Z; ++j)
+                w[((size_t)j * h->Q + m) * P4 * 4 + p] =
+                    (float)h->Sm64[((size_t)m * h->P + p) * h->Z + j];
+    SW_CUDA(cudaMemcpy(h->fft->S4, w.data(), w.size() * sizeof(float), cudaMemcpyHostToDevice));
     return SWOPT_OK;
 }
 

@@ -244,6 +244,9 @@ struct swopt_handle {
     bool capturing = false;
     cudaStream_t cap_stream = nullptr;
     swopt::IterGraph graphs[3];
+    bool cap_valid = false;       // graphs hold iterations captured with the next three
+    swopt_solve_params cap_prm{};
+    double cap_step = 0.0, cap_jstep2 = 0.0;
     uint64_t graph_gen = 0;       // bumped whenever captured work may have gone stale
     std::vector<std::pair<cudaEvent_t, int>> cap_events;
 
@@ -349,7 +352,7 @@ swopt_status tc_supported(swopt_handle* h);
 void fft_prepare(swopt_handle* h);
 bool fft_prepare_bf16(swopt_handle* h);
 void fft_release(swopt_handle* h);
-// After h->Sm has changed (synchronises the device).
+// After h->Sm has changed (with no kernel of the handle in flight).
 swopt_status fft_weights(swopt_handle* h);
 // h->u = (scale ? Cm : 1) A P c - ytil (ytil may be null)
 swopt_status fft_forward(swopt_handle* h, const float* c, const float* ytil, int scale, bool round,
