@@ -299,6 +299,23 @@ bool route_fft(const swopt_handle* h)
     return true;
 }
 
+// SWOPT_PREC_BF16 rounds both operands of a contraction to BF16; the split
+// precisions keep (at least nearly) all of FP32, and FP32 is exact.
+bool rounds(const swopt_handle* h) { return h->precision == SWOPT_PREC_BF16; }
+
+// What the selected precision's route needs (synchronises; never called while
+// capturing).
+swopt_status prepare_route(swopt_handle* h)
+{
+    if (!use_tc(h)) return SWOPT_OK;
+    if (!route_fft(h)) return tc_prepare(h);
+    if (rounds(h) && !fft_prepare_bf16(h)) {
+        set_error("no memory for the spectrum of the BF16 kernel");
+        return SWOPT_ERR_OOM;
+    }
+    return SWOPT_OK;
+}
+
 // The tensor-core operator of the selected precision, built if the spectral
 // kernels do not serve it (synchronises; never called while capturing).
 swopt_status ensure_tc(swopt_handle* h)
@@ -306,10 +323,6 @@ swopt_status ensure_tc(swopt_handle* h)
     if (!use_tc(h) || h->tc) return SWOPT_OK;
     return tc_prepare(h);
 }
-
-// SWOPT_PREC_BF16 rounds both operands of a contraction to BF16; the split
-// precisions keep (at least nearly) all of FP32, and FP32 is exact.
-bool rounds(const swopt_handle* h) { return h->precision == SWOPT_PREC_BF16; }
 
 // P then A.  out = A_OUT_U writes h->u (FP32 [Q][S][Twp]); out = A_OUT_R writes
 // the input format of apply_AT (h->u for the FP32 kernels, the padded BF16
@@ -553,8 +566,7 @@ swopt_status ensure_ref(swopt_handle* h)
     const int rp = h->prm.refine_precision;
     if (h->prm.refine_every <= 0 || rp == SWOPT_PREC_FP32 || rp == h->precision) return SWOPT_OK;
     RefScope sc(h, rp);
-    if (route_fft(h)) return SWOPT_OK;
-    return tc_prepare(h);
+    return prepare_route(h);
 }
 
 // Kind of FISTA iteration number h->iter: 1 when the refined solve
@@ -631,6 +643,21 @@ swopt_status fista_iteration(swopt_handle* h, int kind, cudaStream_t st)
         // both branches are launched behind the gate
         SW_TRY(refine_decide(h, h->tmp, h->c, SC_BUDGET, h->prm.refine_every,
                              h->prm.refine_budget, st));
+        bool one_chain = route_fft(h) && fft_refine_gated(h), round2 = false;
+        if (one_chain) {
+            RefScope r(h, h->prm.refine_precision);
+            round2 = rounds(h);
+            one_chain = route_fft(h);
+        }
+        if (one_chain && (rounds(h) || !round2)) {
+            FftImage img;
+            img.mode = 2;
+            img.alpha = alpha;
+            img.out = h->zin;
+            img.xi = h->xi;
+            img.G = h->G;
+            return fft_refine(h, h->tmp, h->c, h->ytil, rounds(h), round2, img, st);
+        }
         {
             GateScope g0(h, 0);
             SW_TRY(refined_gradient(h, h->tmp, nullptr, 1, st));
@@ -691,10 +718,14 @@ swopt_status build_graph(swopt_handle* h, int kind)
             if (r.first == ev) return r.second;
         return nullptr;
     };
-    for (size_t i = ev0; i + 1 < h->cap_events.size(); ++i) {
+    for (size_t i = ev0; i < h->cap_events.size(); ++i) {
         const auto& b = h->cap_events[i];
-        const auto& en = h->cap_events[i + 1];
-        if (b.second >= 0 && en.second == -1 - b.second) {
+        if (b.second < 0) continue;
+        // its end: the next marker of the same kind (one launch may count as two kinds)
+        size_t j = i + 1;
+        while (j < h->cap_events.size() && h->cap_events[j].second != -1 - b.second) ++j;
+        if (j < h->cap_events.size()) {
+            const auto& en = h->cap_events[j];
             GraphProbe pr;
             pr.begin = node_of(b.first);
             pr.end = node_of(en.first);
@@ -703,7 +734,6 @@ swopt_status build_graph(swopt_handle* h, int kind)
             pr.gated = b.second >= 16;
             pr.kernel = b.second & 15;
             if (pr.begin && pr.end) G.probes.push_back(pr);
-            ++i;
         }
     }
     return SWOPT_OK;
@@ -764,14 +794,16 @@ swopt_status objective_impl(swopt_handle* h, const float* c, const float* y, boo
         SW_TRY(launch_fold(h, y, h->yfold, st));
         SW_TRY(reduce_sumsq(h, y, (size_t)h->N * h->S * h->T, SC_A, st));
     }
-    SW_TRY(reduce_dot(h, h->u, yt, nu_of(h), SC_B, st));
-    SW_TRY(reduce_states(h, h->u, SC_E, st));
-    SW_TRY(reduce_abs(h, c, nc_of(h), SC_C, st));
-    SW_TRY(reduce_tv(h, c, SC_D, st));
+    SumList sums;
+    SW_TRY(sum_dot(h, h->u, yt, nu_of(h), SC_B, &sums, st));
+    SW_TRY(sum_abs(h, c, nc_of(h), SC_C, &sums, st));
+    SW_TRY(sum_tv(h, c, SC_D, &sums, st));
     if (lam_3 != 0.0) {  // sum_n TV((S c)^n) = sum_m Cm TV(S_m c)
         SW_TRY(launch_states(h, c, h->b, st));
-        SW_TRY(reduce_tv_states(h, h->b, SC_F, st));
+        SW_TRY(sum_tv_states(h, h->b, SC_F, &sums, st));
     }
+    SW_TRY(sum_states(h, h->u, SC_E, &sums, st));
+    SW_TRY(finish_sums(h, sums, st));
     SW_TRY(read_scalars(h, st));
     const double* v = h->scal_host;
     const double df = 0.5 * (v[bound ? SC_YSQ : SC_A] + v[SC_E] - 2.0 * v[SC_B]);
@@ -889,7 +921,7 @@ swopt_status swopt_create(const swopt_geometry* geom, const double* K_host,
     step(dalloc(&h->b, nb_of(h)));
     step(dalloc(&h->u, nu_of(h)));
     step(dalloc(&h->g, nb_of(h)));
-    h->red_cap = std::max({4096, simt_forward_blocks(h) + 64, tc_forward_blocks(h) + 64,
+    h->red_cap = std::max({kObjectiveSums, simt_forward_blocks(h) + 64, tc_forward_blocks(h) + 64,
                            h->Q * h->P * h->Z + 64});
     step(dalloc(&h->red, (size_t)h->red_cap));
     step(dalloc(&h->scal, (size_t)SC_COUNT));
@@ -974,12 +1006,8 @@ swopt_status swopt_set_precision(swopt_handle* h, int precision)
         h->precision = precision;
         // a geometry that the tensor-core kernels refuse stays refused
         swopt_status s = tc_supported(h);
-        if (s == SWOPT_OK && rounds(h) && route_fft(h) && !fft_prepare_bf16(h)) {
-            set_error("no memory for the spectrum of the BF16 kernel");
-            s = SWOPT_ERR_OOM;
-        }
         if (s == SWOPT_OK && route_fft(h)) tc_release(h);  // of another precision
-        else if (s == SWOPT_OK) s = tc_prepare(h);
+        if (s == SWOPT_OK) s = prepare_route(h);
         if (s != SWOPT_OK) {
             h->precision = prev;
             return s;
@@ -1719,8 +1747,7 @@ swopt_status swopt_tc_configure(swopt_handle* h, int kernel_id, int tiles_per_ct
     h->tc_force_ra[kernel_id] = accumulators;
     release_ref(h);
     tc_release(h);
-    if (use_tc(h) && !route_fft(h)) return tc_prepare(h);
-    return SWOPT_OK;
+    return prepare_route(h);
 }
 
 swopt_status swopt_tc_config(swopt_handle* h, int kernel_id, int* tiles_per_cta,
@@ -1755,8 +1782,7 @@ swopt_status swopt_tc_schedule(swopt_handle* h, int kernel_id, int split, int bu
     h->tc_force_nbuf[kernel_id] = buffers;
     release_ref(h);
     tc_release(h);
-    if (use_tc(h) && !route_fft(h)) return tc_prepare(h);
-    return SWOPT_OK;
+    return prepare_route(h);
 }
 
 swopt_status swopt_tc_schedule_info(swopt_handle* h, int kernel_id, int* split, int* buffers,

@@ -49,7 +49,7 @@ namespace {
 constexpr int kFB = 8;           // frequencies per block of the spectral product
 constexpr int kOG = 8;           // output channels per group of the banded kernel
 constexpr int kMaxFftThreads = 256;
-constexpr int kSpecThreads = 224;
+constexpr int kSpecThreads = 256;
 constexpr size_t kSpecSmem = 220 * 1024;  // most dynamic shared memory of the product
 
 // ---------------------------------------------------------------------------
@@ -294,12 +294,22 @@ struct FftShape {
     int tiles;      // y.tiles * x.tiles
     int rows_in;    // rows of a tile that hold data before the y transform
     int rows_out;   // rows of a tile that hold results after the inverse y transform
+    // Launches that serve a decision taken on the device (the refined solve's
+    // increment or exact gradient): *sel != 0 takes the arguments marked 2.
+    const int* sel;  // null: no second variant
     int round;      // operands rounded to BF16 (per state)
+    int round2;
     const float* Sm;  // [Q][P][Z]
     const float* Kf;  // [Z][k][k][Twp] FP32 kernel (direct sums of non-finite outputs)
     const int* gate;
     int want;
 };
+
+// True if the launch takes its second variant (after grid_dependency()).
+__device__ __forceinline__ bool second_variant(const FftShape& s)
+{
+    return s.sel != nullptr && *(volatile const int*)s.sel != 0;
+}
 
 __device__ __forceinline__ float round_if(float v, int round)
 {
@@ -330,8 +340,8 @@ __device__ __forceinline__ float folded(const FftShape& s, const float* __restri
 
 // One output of A by its direct sum (the order and the zero blocks of
 // fwd_simt_kernel); only for outputs that the transforms made non-finite.
-__device__ __noinline__ float direct_forward(const FftShape& s, const float* c, int m, int y,
-                                             int x, int w)
+__device__ __noinline__ float direct_forward(const FftShape& s, int round, const float* c, int m,
+                                             int y, int x, int w)
 {
     float acc = 0.f;
     for (int j = 0; j < s.Z; ++j)
@@ -344,15 +354,15 @@ __device__ __noinline__ float direct_forward(const FftShape& s, const float* c, 
                 for (int i = 0; i < 8; ++i) any |= kp[(w & ~7) + i] != 0.f;
                 if (!any) continue;
                 const float b = state_value(s, c, m, (size_t)yy * s.X + xx, j);
-                acc = fmaf(round_if(b, s.round), round_if(kp[w], s.round), acc);
+                acc = fmaf(round_if(b, round), round_if(kp[w], round), acc);
             }
     return acc;
 }
 
 // One output of A^T (state m, depth j) by its direct sum over r, either the
 // residual [Q][Y][X][Twp] or (from_y) the measurements folded on the way.
-__device__ __noinline__ float direct_adjoint(const FftShape& s, const float* r, int from_y, int m,
-                                             int y, int x, int j)
+__device__ __noinline__ float direct_adjoint(const FftShape& s, int round, const float* r,
+                                             int from_y, int m, int y, int x, int j)
 {
     const int j8 = j & ~7;
     float acc = 0.f;
@@ -370,8 +380,7 @@ __device__ __noinline__ float direct_adjoint(const FftShape& s, const float* r, 
                 const size_t pos = (size_t)yy * s.X + xx;
                 const float v = from_y ? folded(s, r, m, pos, w)
                                        : r[((size_t)m * s.Y * s.X + pos) * s.Twp + w];
-                acc = fmaf(round_if(v, s.round), round_if(s.Kf[(size_t)j * kk + tap], s.round),
-                           acc);
+                acc = fmaf(round_if(v, round), round_if(s.Kf[(size_t)j * kk + tap], round), acc);
             }
     return acc;
 }
@@ -381,7 +390,8 @@ __device__ __noinline__ float direct_adjoint(const FftShape& s, const float* r, 
 // lanes are neighbouring channel pairs (then rows, or x frequencies).  Bound by
 // memory: a pass reads and writes every value once.
 // ---------------------------------------------------------------------------
-enum { SRC_C = 0, SRC_STATES = 1, SRC_U = 2, SRC_Y = 3 };
+// SRC_GATED: SRC_STATES, or SRC_C as the second variant
+enum { SRC_C = 0, SRC_STATES = 1, SRC_U = 2, SRC_Y = 3, SRC_GATED = 4 };
 
 struct XForward {
     FftShape s;
@@ -390,6 +400,8 @@ struct XForward {
     int C2;         // channel pairs
     int vec;        // pairs may be read as one float2
     unsigned items; // planes * tiles * rows_in * C2
+    const float* src2;
+    unsigned items2;
 };
 
 template <int SRC>
@@ -401,7 +413,11 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_forward_kernel(const 
     if (gated_off(s.gate, s.want)) return;
     const int lane = threadIdx.x & 31;
     const unsigned item = blockIdx.x * 32u + lane;
-    const bool ok = item < a.items;
+    const bool alt = second_variant(s);
+    const float* src = alt ? a.src2 : a.src;
+    const int round = alt ? s.round2 : s.round;
+    constexpr bool kStates = SRC == SRC_STATES || SRC == SRC_GATED;
+    const bool ok = item < (alt ? a.items2 : a.items);
     const unsigned q = item % (unsigned)a.C2, line = item / (unsigned)a.C2;
     const unsigned row = line % (unsigned)s.rows_in, pt = line / (unsigned)s.rows_in;
     const int tile = (int)(pt % (unsigned)s.tiles), plane = (int)(pt / (unsigned)s.tiles);
@@ -413,12 +429,12 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_forward_kernel(const 
     const size_t row0 = (size_t)(row_ok ? gy : 0) * s.X;
     const bool two = ch + 1 < s.Z;
     // SRC_STATES: this thread's switching weights (its state and depths)
-    float2 wt[SRC == SRC_STATES ? 8 : 1];
-    if (SRC == SRC_STATES) {
+    float2 wt[kStates ? 8 : 1];
+    if (kStates) {
 #pragma unroll
         for (int p = 0; p < 8; ++p) {
             wt[p] = make_float2(0.f, 0.f);
-            if (!ok || p >= s.P) continue;
+            if (!ok || p >= s.P || (SRC == SRC_GATED && alt)) continue;
             const float* sp = s.Sm + ((size_t)plane * s.P + p) * s.Z + ch;
             wt[p].x = __ldg(sp);
             if (two) wt[p].y = __ldg(sp + 1);
@@ -452,29 +468,32 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_forward_kernel(const 
             }
 #pragma unroll
             for (int i = 0; i < R; ++i)
-                v[i] = SRC == SRC_STATES
+                v[i] = kStates
                            ? make_float2(fmaf(w.x, t[i].x, v[i].x), fmaf(w.y, t[i].y, v[i].y))
                            : cadd(v[i], t[i]);
         };
         const ptrdiff_t at = (ptrdiff_t)row0 + first;  // may lie outside; guarded by inside()
         const float2 none = make_float2(0.f, 0.f);
         if (SRC == SRC_C) {
-            add(a.src + ((ptrdiff_t)(plane * YX) + at) * s.Z + ch, (size_t)R2 * s.Z, two, none);
-        } else if (SRC == SRC_STATES) {
+            add(src + ((ptrdiff_t)(plane * YX) + at) * s.Z + ch, (size_t)R2 * s.Z, two, none);
+        } else if (SRC == SRC_GATED && alt) {
+            add(src + ((ptrdiff_t)(plane * YX) + at) * s.Z + ch, (size_t)R2 * s.Z, two,
+                make_float2(1.f, 1.f));
+        } else if (kStates) {
 #pragma unroll
             for (int p = 0; p < 8; ++p)
                 if (p < s.P)
-                    add(a.src + ((ptrdiff_t)(p * YX) + at) * s.Z + ch, (size_t)R2 * s.Z, two, wt[p]);
+                    add(src + ((ptrdiff_t)(p * YX) + at) * s.Z + ch, (size_t)R2 * s.Z, two, wt[p]);
         } else if (SRC == SRC_U) {
-            add(a.src + ((ptrdiff_t)(plane * YX) + at) * s.Twp + ch, (size_t)R2 * s.Twp, true, none);
+            add(src + ((ptrdiff_t)(plane * YX) + at) * s.Twp + ch, (size_t)R2 * s.Twp, true, none);
         } else {
             const int t = s.t0 + ch;
             if (t < s.T)
                 for (int n = plane; n < s.N; n += s.ncyc)
-                    add(a.src + ((ptrdiff_t)(n * YX) + at) * s.T + t, (size_t)R2 * s.T, t + 1 < s.T,
+                    add(src + ((ptrdiff_t)(n * YX) + at) * s.T + t, (size_t)R2 * s.T, t + 1 < s.T,
                         none);
         }
-        if (SRC != SRC_C && s.round) {
+        if (SRC != SRC_C && round) {
 #pragma unroll
             for (int i = 0; i < R; ++i) v[i] = make_float2(round_if(v[i].x, 1), round_if(v[i].y, 1));
         }
@@ -494,6 +513,7 @@ struct YPass {
     float2* out;        // forward: [plane tile][Ly][Lx][C2]; inverse: [..][rows_out][Lx][C2]
     unsigned width;     // Lx * C2
     unsigned items;     // plane-tiles * width
+    unsigned items2;
 };
 
 template <int S>
@@ -504,7 +524,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_y_kernel(const YPass a)
     grid_dependency();
     if (gated_off(s.gate, s.want)) return;
     const unsigned item = blockIdx.x * 32u + (threadIdx.x & 31);
-    const bool ok = item < a.items;
+    const bool ok = item < (second_variant(s) ? a.items2 : a.items);
     const unsigned col = item % a.width, pt = item / a.width;
     const int rows = S < 0 ? s.rows_in : s.y.L;
     const float2* in = a.in + (size_t)pt * rows * a.width + col;
@@ -554,13 +574,13 @@ struct XInverse {
     const float* Cmf;   // null: no scale
     const float* c;     // input of A (direct sums)
     // images: IMG_STORE out = v; IMG_STEP out = xi - alpha v; IMG_REFINE as pt_refine_kernel
-    int add;
+    int add, add2;
     float alpha;
     const float* xi;
     float* G;
     const double* scal;
     const float* r;     // input of A^T (direct sums): residual or measurements
-    int keep;           // whether r holds them (KEEP_*)
+    int keep, keep2;    // whether r holds them (KEEP_*)
     const double* ysq;
     int from_y;
     int per_state;      // planes are states (else species, summed over the states)
@@ -585,6 +605,7 @@ __device__ __noinline__ void fix_image(const XInverse& a, float2* slot, int R, i
                                        int gx0, int gy, int plane, int ch)
 {
     const FftShape& s = a.s;
+    const int round = second_variant(s) ? s.round2 : s.round;
     for (int i = 0; i < R; ++i) {
         const int o = k1 + R1 * i - s.x.pad, gx = gx0 + o;
         if (o < 0 || o >= s.x.out || gx >= s.X) continue;
@@ -593,11 +614,11 @@ __device__ __noinline__ void fix_image(const XInverse& a, float2* slot, int R, i
             if (isfinite(*p)) continue;
             float acc = 0.f;
             if (a.per_state) {
-                acc = direct_adjoint(s, a.r, a.from_y, plane, gy, gx, ch + h);
+                acc = direct_adjoint(s, round, a.r, a.from_y, plane, gy, gx, ch + h);
             } else {
                 for (int m = 0; m < s.Q; ++m)
                     acc = fmaf(s.Sm[((size_t)m * s.P + plane) * s.Z + ch + h],
-                               direct_adjoint(s, a.r, a.from_y, m, gy, gx, ch + h), acc);
+                               direct_adjoint(s, round, a.r, a.from_y, m, gy, gx, ch + h), acc);
             }
             *p = acc;
         }
@@ -605,15 +626,15 @@ __device__ __noinline__ void fix_image(const XInverse& a, float2* slot, int R, i
 }
 
 // The same for a line of u: columns x0 + k1 + R1 i.
-__device__ __noinline__ void fix_u(const FftShape& s, const float* c, float2* slot, int R, int k1,
-                                   int R1, int x0, int end, int gy, int m, int w)
+__device__ __noinline__ void fix_u(const FftShape& s, int round, const float* c, float2* slot, int R,
+                                   int k1, int R1, int x0, int end, int gy, int m, int w)
 {
     for (int i = 0; i < R; ++i) {
         const int gx = x0 + k1 + R1 * i;
         if (gx < max(0, x0 + s.x.pad) || gx >= end) continue;
         for (int h = 0; h < 2; ++h) {
             float* p = reinterpret_cast<float*>(slot + i * 32) + h;
-            if (!isfinite(*p)) *p = direct_forward(s, c, m, gy, gx, w + h);
+            if (!isfinite(*p)) *p = direct_forward(s, round, c, m, gy, gx, w + h);
         }
     }
 }
@@ -638,6 +659,8 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
     const size_t YX = (size_t)s.Y * s.X;
     const float2* in = a.in + (size_t)line * s.x.L * a.C2 + q;
     const float beta = MODE == IMG_REFINE ? (float)a.scal[1] : 0.f;
+    const bool alt = second_variant(s);
+    const int add = alt ? a.add2 : a.add, keep = alt ? a.keep2 : a.keep;
     const bool two = ch + 1 < s.Z;
     fft_line<1>(
         s.x, sm,
@@ -654,7 +677,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
                 const int o = k1 + R1 * i - s.x.pad, gx = gx0 + o;
                 return o >= 0 && o < s.x.out && gx < s.X ? gx : -1;
             };
-            if (any_nonfinite(v) && kept(a.keep, a.ysq)) {
+            if (any_nonfinite(v) && kept(keep, a.ysq)) {
                 float2* slot = sm + k1 * R * 32 + (threadIdx.x & 31);
                 through_slots(v, slot, [&] { fix_image(a, slot, R, k1, R1, gx0, gy, plane, ch); });
             }
@@ -690,7 +713,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
                     if (gx < 0) continue;
                     float2 g = v[b + i];
                     if (MODE == IMG_REFINE) {
-                        if (a.add) g = cadd(go[i], g);
+                        if (add) g = cadd(go[i], g);
                         put(a.G + at(gx), g);
                         g = make_float2(fmaf(beta, g.x - go[i].x, g.x),
                                         fmaf(beta, g.y - go[i].y, g.y));
@@ -750,7 +773,8 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_u_kernel(const XInver
             if (any_nonfinite(v)) {
                 float2* slot = sm + k1 * R * 32 + (threadIdx.x & 31);
                 through_slots(v, slot, [&] {
-                    fix_u(s, a.c, slot, R, k1, R1, gx0 - s.x.pad, min(s.X, gx0 + s.x.out), gy, m, w);
+                    fix_u(s, s.round, a.c, slot, R, k1, R1, gx0 - s.x.pad, min(s.X, gx0 + s.x.out), gy,
+                          m, w);
                 });
             }
 #pragma unroll
@@ -780,6 +804,9 @@ struct XResidual {
     float* u;
     int keep;           // KEEP_*
     const double* ysq;  // KEEP_NONFINITE: sum of squares of the measurements
+    const float* ytil2;
+    const float* c2;
+    int keep2;
 };
 
 // 112 registers: three blocks of 6 warps per SM, without spills
@@ -799,7 +826,10 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
     const float2* in = a.in + (size_t)line * ax.L * a.C2 + q;
     float2* out = a.out + (size_t)line * ax.L * a.C2 + q;
     const float cm = ok ? a.Cmf[m] : 1.f;
-    const bool keep = kept(a.keep, a.ysq);
+    const bool alt = second_variant(s);
+    const float* ytil = alt ? a.ytil2 : a.ytil;
+    const int round = alt ? s.round2 : s.round;
+    const bool keep = kept(alt ? a.keep2 : a.keep, a.ysq);
     const size_t base = (((size_t)m * s.Y + row) * s.X) * s.Twp + w;
     auto load = [&](auto& v, int n2, int R2) {
         constexpr int R = sizeof(v) / sizeof(v[0]);
@@ -819,13 +849,13 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
 #pragma unroll
         for (int i = 0; i < R; ++i) {
             const int gx = k1 + R1 * i;
-            yt[i] = a.ytil && ok && gx < s.X ? load_produced(reinterpret_cast<const float2*>(
-                                                   a.ytil + base + (size_t)gx * s.Twp))
+            yt[i] = ytil && ok && gx < s.X ? load_produced(reinterpret_cast<const float2*>(
+                                                   ytil + base + (size_t)gx * s.Twp))
                                              : make_float2(0.f, 0.f);
         }
         if (ok && any_nonfinite(v)) {
             float2* slot = sm + k1 * R * 32 + lane;
-            through_slots(v, slot, [&] { fix_u(s, a.c, slot, R, k1, R1, 0, s.X, row, m, w); });
+            through_slots(v, slot, [&] { fix_u(s, round, alt ? a.c2 : a.c, slot, R, k1, R1, 0, s.X, row, m, w); });
         }
 #pragma unroll
         for (int i = 0; i < R; ++i) {
@@ -833,7 +863,7 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
             v[i] = make_float2(fmaf(cm, v[i].x, -yt[i].x), fmaf(cm, v[i].y, -yt[i].y));
             if (keep && ok && gx < s.X)
                 *reinterpret_cast<float2*>(a.u + base + (size_t)gx * s.Twp) = v[i];
-            if (s.round) v[i] = make_float2(round_if(v[i].x, 1), round_if(v[i].y, 1));
+            if (round) v[i] = make_float2(round_if(v[i].x, 1), round_if(v[i].y, 1));
             if (gx >= s.X) v[i] = make_float2(0.f, 0.f);
         }
         Dft<R, -1>::run(v);
@@ -890,6 +920,7 @@ struct Spec {
     const float2* in;      // [plane][tile][Ly][Lx][in_C2]
     float2* out;           // [plane][tile][Ly][Lx][out_C2]
     const float4* K;       // [freq block][row][kFB][kOG / 2] (two channels each)
+    const float4* K2;
     const int4* tab;       // per group: first row, first contracted channel, their count
     const float4* S4;      // [Z][Q][species in fours]
     int groups;
@@ -932,7 +963,11 @@ __host__ __device__ constexpr size_t spec_smem(int MC, int pairs, int warps)
            (size_t)warps * kRingSlots * kRingRows * 512;
 }
 
-template <int MC, bool ADJ, bool FUSED>
+// MAP: how P (or P^T) takes part.  MAP_NONE: the planes are states; MAP_SPECIES:
+// they are species; MAP_GATED: states, or species as the second variant (A).
+enum { MAP_NONE = 0, MAP_SPECIES = 1, MAP_GATED = 2 };
+
+template <int MC, bool ADJ, int MAP>
 __global__ void __launch_bounds__(kSpecThreads, 2) spec_kernel(const Spec a)
 {
     extern __shared__ float4 sm4[];
@@ -943,12 +978,15 @@ __global__ void __launch_bounds__(kSpecThreads, 2) spec_kernel(const Spec a)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int Lx = s.x.L, Ly = s.y.L;
     const size_t area = (size_t)Ly * Lx;
-    const int loops = ADJ && FUSED ? a.chunks : 1;
-    const int tile = ADJ && FUSED ? (int)blockIdx.y : (int)blockIdx.y / a.chunks;
-    const int chunk0 = ADJ && FUSED ? 0 : (int)blockIdx.y % a.chunks;
+    const bool alt = second_variant(s);
+    const bool species = MAP == MAP_GATED ? alt : MAP == MAP_SPECIES;
+    constexpr bool kFuseT = ADJ && MAP == MAP_SPECIES;
+    const int loops = kFuseT ? a.chunks : 1;
+    const int tile = kFuseT ? (int)blockIdx.y : (int)blockIdx.y / a.chunks;
+    const int chunk0 = kFuseT ? 0 : (int)blockIdx.y % a.chunks;
     const int P4 = (s.P + 3) / 4;
     float4* ring = sm4 + (size_t)2 * a.in_C2 * kFB * MS2 + warp * (kRingSlots * kRingRows * 32) + lane;
-    const float4* kblk = a.K + (size_t)blockIdx.x * a.rows * (kFB * kOG / 2) + lane;
+    const float4* kblk = (alt ? a.K2 : a.K) + (size_t)blockIdx.x * a.rows * (kFB * kOG / 2) + lane;
 
     auto locate = [&](int f, size_t* at, size_t* mirror) -> bool {
         const int id = (int)blockIdx.x * kFB + f;
@@ -1009,7 +1047,7 @@ __global__ void __launch_bounds__(kSpecThreads, 2) spec_kernel(const Spec a)
                     x0 = make_float2(z.x + zm.x, z.y - zm.y);
                     x1 = make_float2(z.y + zm.y, zm.x - z.x);
                 };
-                if (!ADJ && FUSED) {
+                if (!ADJ && MAP != MAP_NONE && species) {
                     for (int p4 = 0; p4 < P4; ++p4) {
                         float2 x0[4], x1[4];
 #pragma unroll
@@ -1123,7 +1161,7 @@ __global__ void __launch_bounds__(kSpecThreads, 2) spec_kernel(const Spec a)
                 o[at * a.out_C2] = w;
                 if (mi != at) o[mi * a.out_C2] = wm;
             };
-            if (ADJ && FUSED) {
+            if (kFuseT) {
                 for (int p4 = 0; p4 < P4; ++p4) {
                     const float4* w0 = a.S4 + ((size_t)(2 * oq) * s.Q + m0) * P4 + p4;
                     const float4* w1 = 2 * oq + 1 < s.Z ? w0 + (size_t)s.Q * P4 : w0;
@@ -1348,15 +1386,23 @@ long long band_table(const std::vector<int>& lo, const std::vector<int>& hi, int
     return rows;
 }
 
+// Warps of a block: the fewest rounds of up to 8 over the groups, evenly filled
+// (9 groups on 7 warps took two rounds of which one held 2 groups).
+int spec_warps(int groups)
+{
+    const int rounds = (groups + kSpecThreads / 32 - 1) / (kSpecThreads / 32);
+    return std::max(1, (groups + rounds - 1) / std::max(1, rounds));
+}
+
 // States per block: an even count up to 10, the fewest reads of K^ first, then
 // the fewest padding states; blocks that leave room for two per SM where
 // possible (0: none fits).
-int pick_chunk(int Q, int pairs)
+int pick_chunk(int Q, int pairs, int warps)
 {
     for (size_t cap : {(size_t)112 * 1024, kSpecSmem}) {
         int best = 0, least = 1 << 30;
         for (int mc = 10; mc >= 2; mc -= 2) {
-            if (spec_smem(mc, pairs, kSpecThreads / 32) > cap) continue;
+            if (spec_smem(mc, pairs, warps) > cap) continue;
             const int blocks = (Q + mc - 1) / mc, cost = blocks * (64 + mc);
             if (cost < least) {
                 least = cost;
@@ -1471,7 +1517,8 @@ void fft_prepare(swopt_handle* h)
     const long long frows = band_table(wlo, whi, tw, &ft);
     const long long arows = band_table(jlo, jhi, h->Z, &at);
     const int Cz2 = (h->Z + 1) / 2, Ct2 = (tw + 1) / 2;
-    const int fchunk = pick_chunk(h->Q, Cz2), achunk = pick_chunk(h->Q, Ct2);
+    const int fchunk = pick_chunk(h->Q, Cz2, spec_warps((int)ft.size()));
+    const int achunk = pick_chunk(h->Q, Ct2, spec_warps((int)at.size()));
     if (!fchunk || !achunk) return;
 
     // lengths: the least estimated time over all pairs (K^ and the spectra through
@@ -1568,7 +1615,8 @@ FftShape shape_of(const swopt_handle* h, bool round)
     s.Y = h->Y; s.X = h->X; s.Z = h->Z; s.T = h->T; s.N = h->N; s.P = h->P; s.Q = h->Q;
     s.ncyc = h->ncyc; s.Twp = h->Twp; s.t0 = h->t0; s.k = h->k; s.r = h->r;
     s.tiles = f->tiles; s.rows_in = f->rows_in; s.rows_out = f->rows_out;
-    s.round = round ? 1 : 0;
+    s.sel = nullptr;
+    s.round = s.round2 = round ? 1 : 0;
     s.Sm = h->Sm; s.Kf = h->Kf;
     s.gate = h->gate; s.want = h->gate_want;
     return s;
@@ -1590,7 +1638,7 @@ swopt_status launch_lines(swopt_handle* h, void (*kernel)(const Args), const Arg
     return SWOPT_OK;
 }
 
-swopt_status launch_y(swopt_handle* h, const FftShape& s, bool inverse, int planes, int C2,
+swopt_status launch_y(swopt_handle* h, const FftShape& s, bool inverse, int planes, int planes2, int C2,
                       const float2* in, float2* out, cudaStream_t st)
 {
     YPass a{};
@@ -1599,28 +1647,29 @@ swopt_status launch_y(swopt_handle* h, const FftShape& s, bool inverse, int plan
     a.out = out;
     a.width = (unsigned)(s.x.L * C2);
     a.items = (unsigned)(planes * s.tiles) * a.width;
+    a.items2 = (unsigned)(planes2 * s.tiles) * a.width;
     return launch_lines(h, inverse ? fft_y_kernel<1> : fft_y_kernel<-1>, a, s.y, st);
 }
 
-template <int MC, bool ADJ, bool FUSED>
+template <int MC, bool ADJ, int MAP>
 swopt_status launch_spec_mc(swopt_handle* h, const Spec& a, cudaStream_t st)
 {
-    auto kernel = spec_kernel<MC, ADJ, FUSED>;
-    const int warps = std::min(kSpecThreads / 32, std::max(1, a.groups));
+    auto kernel = spec_kernel<MC, ADJ, MAP>;
+    const int warps = spec_warps(a.groups);
     const size_t smem = spec_smem(MC, a.in_C2, warps);
     if (smem > 48 * 1024)
         SW_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSpecSmem));
     const dim3 grid((unsigned)h->fft->blocks,
-                    (unsigned)(a.s.tiles * (ADJ && FUSED ? 1 : a.chunks)));
+                    (unsigned)(a.s.tiles * (ADJ && MAP == MAP_SPECIES ? 1 : a.chunks)));
     SW_CUDA(launch_pdl(kernel, grid, 32 * warps, smem, st, a));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
 
-template <bool ADJ, bool FUSED>
+template <bool ADJ, int MAP>
 swopt_status launch_spec(swopt_handle* h, const FftShape& s, const float2* in, float2* out,
-                         int which, cudaStream_t st)
+                         cudaStream_t st)
 {
     const FftOperator* f = h->fft;
     const int mc = ADJ ? f->achunk : f->fchunk;
@@ -1628,7 +1677,12 @@ swopt_status launch_spec(swopt_handle* h, const FftShape& s, const float2* in, f
     a.s = s;
     a.in = in;
     a.out = out;
-    a.K = reinterpret_cast<const float4*>(ADJ ? f->KA[which] : f->KF[which]);
+    a.K = reinterpret_cast<const float4*>(ADJ ? f->KA[s.round] : f->KF[s.round]);
+    a.K2 = reinterpret_cast<const float4*>(ADJ ? f->KA[s.round2] : f->KF[s.round2]);
+    if (!a.K || !a.K2) {
+        set_error("internal: no spectrum of the kernel for the selected precision");
+        return SWOPT_ERR_DEVICE_CHECK;
+    }
     a.tab = ADJ ? f->atab : f->ftab;
     a.groups = ADJ ? f->agroups : f->fgroups;
     a.rows = ADJ ? f->arows : f->frows;
@@ -1638,11 +1692,11 @@ swopt_status launch_spec(swopt_handle* h, const FftShape& s, const float2* in, f
     a.hx = f->hx;
     a.S4 = f->S4;
     switch (mc) {
-    case 2: return launch_spec_mc<2, ADJ, FUSED>(h, a, st);
-    case 4: return launch_spec_mc<4, ADJ, FUSED>(h, a, st);
-    case 6: return launch_spec_mc<6, ADJ, FUSED>(h, a, st);
-    case 8: return launch_spec_mc<8, ADJ, FUSED>(h, a, st);
-    default: return launch_spec_mc<10, ADJ, FUSED>(h, a, st);
+    case 2: return launch_spec_mc<2, ADJ, MAP>(h, a, st);
+    case 4: return launch_spec_mc<4, ADJ, MAP>(h, a, st);
+    case 6: return launch_spec_mc<6, ADJ, MAP>(h, a, st);
+    case 8: return launch_spec_mc<8, ADJ, MAP>(h, a, st);
+    default: return launch_spec_mc<10, ADJ, MAP>(h, a, st);
     }
 }
 
@@ -1650,37 +1704,46 @@ swopt_status launch_spec(swopt_handle* h, const FftShape& s, const float2* in, f
 
 namespace {
 
-// c -> the spectra of the state images' A, transformed back along y, in f->w1.
-swopt_status forward_to_lines(swopt_handle* h, const FftShape& s, const float* c, cudaStream_t st)
+// c (c2 in the second variant) -> the spectra of the state images' A, transformed
+// back along y, in f->w1.
+swopt_status forward_to_lines(swopt_handle* h, const FftShape& s, const float* c, const float* c2,
+                              cudaStream_t st)
 {
     FftOperator* f = h->fft;
-    const int planes = s.round ? h->Q : h->P;
+    const int planes = s.round ? h->Q : h->P, planes2 = s.round2 ? h->Q : h->P;
+    const unsigned per = (unsigned)(f->tiles * f->rows_in * f->Cz2);
     XForward a{};
     a.s = s;
     a.src = c;
+    a.src2 = c2;
     a.out = f->w0;
     a.C2 = f->Cz2;
-    a.vec = (h->Z % 2) == 0 && aligned8(c);
-    a.items = (unsigned)(planes * f->tiles * f->rows_in * f->Cz2);
-    SW_TRY(launch_lines(h, s.round ? fft_x_forward_kernel<SRC_STATES> : fft_x_forward_kernel<SRC_C>,
+    a.vec = (h->Z % 2) == 0 && aligned8(c) && aligned8(c2);
+    a.items = (unsigned)planes * per;
+    a.items2 = (unsigned)planes2 * per;
+    const bool gated = s.round != s.round2;  // states first, species second
+    SW_TRY(launch_lines(h,
+                        gated     ? fft_x_forward_kernel<SRC_GATED>
+                        : s.round ? fft_x_forward_kernel<SRC_STATES>
+                                  : fft_x_forward_kernel<SRC_C>,
                         a, f->x, st));
-    SW_TRY(launch_y(h, s, false, planes, f->Cz2, f->w0, f->w1, st));
-    if (s.round) SW_TRY((launch_spec<false, false>(h, s, f->w1, f->w0, 1, st)));
-    else SW_TRY((launch_spec<false, true>(h, s, f->w1, f->w0, 0, st)));
-    return launch_y(h, s, true, h->Q, f->Ct2, f->w0, f->w1, st);
+    SW_TRY(launch_y(h, s, false, planes, planes2, f->Cz2, f->w0, f->w1, st));
+    if (gated) SW_TRY((launch_spec<false, MAP_GATED>(h, s, f->w1, f->w0, st)));
+    else if (s.round) SW_TRY((launch_spec<false, MAP_NONE>(h, s, f->w1, f->w0, st)));
+    else SW_TRY((launch_spec<false, MAP_SPECIES>(h, s, f->w1, f->w0, st)));
+    return launch_y(h, s, true, h->Q, h->Q, f->Ct2, f->w0, f->w1, st);
 }
 
 // The lines of A^T's input, transformed along x in f->w0 -> the image outputs.
 swopt_status adjoint_from_lines(swopt_handle* h, const FftShape& s, const float* r, bool from_y,
-                                int keep, const FftImage& img, cudaStream_t st)
+                                int keep, int keep2, const FftImage& img, cudaStream_t st)
 {
     FftOperator* f = h->fft;
-    SW_TRY(launch_y(h, s, false, h->Q, f->Ct2, f->w0, f->w1, st));
-    const int which = s.round ? 1 : 0;
-    if (img.per_state) SW_TRY((launch_spec<true, false>(h, s, f->w1, f->w0, which, st)));
-    else SW_TRY((launch_spec<true, true>(h, s, f->w1, f->w0, which, st)));
+    SW_TRY(launch_y(h, s, false, h->Q, h->Q, f->Ct2, f->w0, f->w1, st));
+    if (img.per_state) SW_TRY((launch_spec<true, MAP_NONE>(h, s, f->w1, f->w0, st)));
+    else SW_TRY((launch_spec<true, MAP_SPECIES>(h, s, f->w1, f->w0, st)));
     const int planes = img.per_state ? h->Q : h->P;
-    SW_TRY(launch_y(h, s, true, planes, f->Cz2, f->w0, f->w1, st));
+    SW_TRY(launch_y(h, s, true, planes, planes, f->Cz2, f->w0, f->w1, st));
     XInverse v{};
     v.s = s;
     v.in = f->w1;
@@ -1688,12 +1751,14 @@ swopt_status adjoint_from_lines(swopt_handle* h, const FftShape& s, const float*
     v.items = (unsigned)(planes * f->tiles * f->rows_out * f->Cz2);
     v.out = img.out;
     v.add = img.add;
+    v.add2 = img.add2;
     v.alpha = img.alpha;
     v.xi = img.xi;
     v.G = img.G;
     v.scal = h->scal;
     v.r = r;
     v.keep = keep;
+    v.keep2 = keep2;
     v.ysq = h->scal + kScalYsq;
     v.from_y = from_y ? 1 : 0;
     v.per_state = img.per_state ? 1 : 0;
@@ -1714,7 +1779,7 @@ swopt_status fft_forward(swopt_handle* h, const float* c, const float* ytil, int
     const FftShape s = shape_of(h, round);
     ProfileRec rec;
     prof_begin(h, 0, st, &rec);
-    SW_TRY(forward_to_lines(h, s, c, st));
+    SW_TRY(forward_to_lines(h, s, c, c, st));
     XInverse v{};
     v.s = s;
     v.in = f->w1;
@@ -1746,48 +1811,112 @@ swopt_status fft_adjoint(swopt_handle* h, const float* src, bool from_y, bool ro
     prof_begin(h, 1, st, &rec);
     SW_TRY(launch_lines(h, from_y ? fft_x_forward_kernel<SRC_Y> : fft_x_forward_kernel<SRC_U>, a,
                         f->x, st));
-    SW_TRY(adjoint_from_lines(h, s, src, from_y, KEEP_ALWAYS, img, st));
+    SW_TRY(adjoint_from_lines(h, s, src, from_y, KEEP_ALWAYS, KEEP_ALWAYS, img, st));
     prof_end(h, &rec, st);
     return SWOPT_OK;
 }
 
+namespace {
+
+int keep_of(FftKeep k)
+{
+    return k == FftKeep::always ? KEEP_ALWAYS : k == FftKeep::never ? KEEP_NEVER : KEEP_NONFINITE;
+}
+
+// From the lines of A in f->w1 through the residual to A^T's output.
+swopt_status residual_to_image(swopt_handle* h, const FftShape& s, const XResidual& args,
+                               const FftImage& img, cudaStream_t st)
+{
+    FftOperator* f = h->fft;
+    XResidual v = args;
+    v.s = s;
+    v.in = f->w1;
+    v.out = f->w0;
+    v.C2 = f->Ct2;
+    v.items = (unsigned)(h->Q * h->Y * f->Ct2);
+    v.Cmf = h->Cmf;
+    v.u = h->u;
+    v.ysq = h->scal + kScalYsq;
+    const size_t smem = (size_t)f->x.L * 32 * sizeof(float2);
+    if (smem > 48 * 1024)
+        SW_CUDA(cudaFuncSetAttribute(fft_x_residual_kernel,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    // nine sub-transforms a pass: one round of nine warps
+    const int warps = std::max(f->x.R1, f->x.R2) == 9 ? 9 : fft_warps(f->x);
+    SW_CUDA(launch_pdl(fft_x_residual_kernel, (v.items + 31) / 32, 32 * warps, smem, st, v));
+    SW_LAUNCHED(h);
+    return adjoint_from_lines(h, s, h->u, false, v.keep, v.keep2, img, st);
+}
+
+}  // namespace
+
 swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool round, FftKeep keep,
                         const FftImage& img, cudaStream_t st)
 {
-    FftOperator* f = h->fft;
-    const size_t smem = (size_t)f->x.L * 32 * sizeof(float2);
-    if (f->tiles > 1) {
+    if (h->fft->tiles > 1) {
         SW_TRY(fft_forward(h, c, ytil, 1, round, st));
         return fft_adjoint(h, h->u, false, round, img, st);
     }
     const FftShape s = shape_of(h, round);
     ProfileRec rec;
     prof_begin(h, 0, st, &rec);
-    SW_TRY(forward_to_lines(h, s, c, st));
+    SW_TRY(forward_to_lines(h, s, c, c, st));
     prof_end(h, &rec, st);
-    XResidual v{};
-    v.s = s;
-    v.in = f->w1;
-    v.out = f->w0;
-    v.C2 = f->Ct2;
-    v.items = (unsigned)(h->Q * h->Y * f->Ct2);
-    v.ytil = ytil;
-    v.Cmf = h->Cmf;
-    v.c = c;
-    v.u = h->u;
-    v.keep = keep == FftKeep::always ? KEEP_ALWAYS
-             : keep == FftKeep::never ? KEEP_NEVER
-                                      : KEEP_NONFINITE;
-    v.ysq = h->scal + kScalYsq;
     prof_begin(h, 1, st, &rec);
-    if (smem > 48 * 1024)
-        SW_CUDA(cudaFuncSetAttribute(fft_x_residual_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    SW_CUDA(launch_pdl(fft_x_residual_kernel, (v.items + 31) / 32, 32 * fft_warps(f->x), smem, st,
-                       v));
-    SW_LAUNCHED(h);
-    SW_TRY(adjoint_from_lines(h, s, h->u, false, v.keep, img, st));
+    XResidual v{};
+    v.ytil = v.ytil2 = ytil;
+    v.c = v.c2 = c;
+    v.keep = v.keep2 = keep_of(keep);
+    SW_TRY(residual_to_image(h, s, v, img, st));
     prof_end(h, &rec, st);
+    return SWOPT_OK;
+}
+
+bool fft_refine_gated(const swopt_handle* h) { return h->fft->tiles == 1; }
+
+swopt_status fft_refine(swopt_handle* h, const float* delta, const float* c, const float* ytil,
+                        bool round, bool round2, const FftImage& image, cudaStream_t st)
+{
+    FftShape s = shape_of(h, round);
+    s.sel = h->sched;
+    s.round2 = round2 ? 1 : 0;
+    FftImage img = image;
+    img.add = 1;
+    img.add2 = 0;
+    // the launches count as the increment's or the exact gradient's, as decided
+    ProfileRec r0, r2;
+    auto gated = [&](auto f) {
+        const int* g = h->gate;
+        h->gate = h->sched;
+        f();
+        h->gate = g;
+    };
+    auto begin = [&](int kernel) {
+        gated([&] {
+            prof_begin(h, kernel, st, &r0);
+            h->in_ref = true;
+            prof_begin(h, kernel, st, &r2);
+            h->in_ref = false;
+        });
+    };
+    auto end = [&] {
+        gated([&] {
+            prof_end(h, &r0, st);
+            prof_end(h, &r2, st);
+        });
+    };
+    begin(0);
+    SW_TRY(forward_to_lines(h, s, delta, c, st));
+    end();
+    begin(1);
+    XResidual v{};
+    v.ytil2 = ytil;
+    v.c = delta;
+    v.c2 = c;
+    v.keep = KEEP_NEVER;
+    v.keep2 = KEEP_NONFINITE;
+    SW_TRY(residual_to_image(h, s, v, img, st));
+    end();
     return SWOPT_OK;
 }
 

@@ -303,22 +303,46 @@ __global__ void expand_kernel(const float* u, float* y, int N, int S,
     }
 }
 
-// ytil[m][s][w] = sum_{n : n mod ncyc = m} y[n][s][t0 + w]  (0 beyond T)
+// ytil[m][s][w] = sum_{n : n mod ncyc = m} y[n][s][t0 + w]  (0 beyond T).  A warp
+// takes rows (m, s), VEC samples per lane and load (4 where T is a multiple of 4
+// and y 16-byte aligned).  40 x 64^2 x 256: 36 us with 64-bit divisions per
+// element, bound by its 63 MB at a quarter of that.
+template <int VEC>
 __global__ void fold_kernel(const float* __restrict__ y, float* __restrict__ ytil, int N, int Q,
                             int S, int T, int ncyc, int t0, int Twp)
 {
-    const size_t n = (size_t)Q * S * Twp;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int w = (int)(i % Twp);
-        const size_t rest = i / Twp;
-        const size_t s = rest % S;
-        const int m = (int)(rest / S);
-        const int t = t0 + w;
-        float acc = 0.f;
-        if (t < T)
-            for (int pn = m; pn < N; pn += ncyc) acc += y[((size_t)pn * S + s) * T + t];
-        ytil[i] = acc;
+    const int lane = threadIdx.x & 31;
+    const unsigned warps = gridDim.x * (blockDim.x >> 5);
+    for (size_t row = blockIdx.x * (size_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+         row < (size_t)Q * S; row += warps) {
+        const int m = (int)(row / (unsigned)S);
+        const size_t s = row - (size_t)m * S;
+        for (int w = VEC * lane; w < Twp; w += 32 * VEC) {
+            const float* src = y + ((size_t)m * S + s) * T + t0 + w;
+            const size_t step = (size_t)ncyc * S * T;
+            float* dst = ytil + row * Twp + w;
+            if (VEC == 4) {
+                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (t0 + w < T) {
+#pragma unroll 4
+                    for (int n = m; n < N; n += ncyc, src += step) {
+                        const float4 v = __ldg(reinterpret_cast<const float4*>(src));
+                        acc.x += v.x;
+                        acc.y += v.y;
+                        acc.z += v.z;
+                        acc.w += v.w;
+                    }
+                }
+                *reinterpret_cast<float4*>(dst) = acc;
+            } else {
+                float acc = 0.f;
+                if (t0 + w < T) {
+#pragma unroll 4
+                    for (int n = m; n < N; n += ncyc, src += step) acc += __ldg(src);
+                }
+                *dst = acc;
+            }
+        }
     }
 }
 
@@ -460,10 +484,10 @@ swopt_status launch_expand(swopt_handle* h, const float* u, float* y, cudaStream
 
 swopt_status launch_fold(swopt_handle* h, const float* y, float* ytil, cudaStream_t st)
 {
-    const size_t n = nu_of(h);
-    int grid = grid_for(n, 256);
-    if (grid > 152 * 32) grid = 152 * 32;
-    fold_kernel<<<grid, 256, 0, st>>>(y, ytil, h->N, h->Q, h->S, h->T, h->ncyc, h->t0, h->Twp);
+    const int grid = std::min(grid_for((size_t)h->Q * h->S, 8), 152 * 16);
+    const bool vec = h->T % 4 == 0 && ((uintptr_t)y & 15u) == 0;
+    (vec ? fold_kernel<4> : fold_kernel<1>)<<<grid, 256, 0, st>>>(y, ytil, h->N, h->Q, h->S, h->T,
+                                                                   h->ncyc, h->t0, h->Twp);
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }

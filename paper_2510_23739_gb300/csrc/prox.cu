@@ -14,7 +14,6 @@
 namespace swopt {
 namespace {
 
-constexpr int kRedBlocks = 1024;
 constexpr int kRedThreads = 256;
 
 __device__ __forceinline__ float clampf(float v, float lo, float hi)
@@ -913,55 +912,75 @@ __global__ void red_tv_weighted_kernel(const float* __restrict__ x, Vol v,
     if (threadIdx.x == 0) parts[blockIdx.x] = s;
 }
 
-__global__ void red_final_kernel(const double* parts, int count, double* out)
+// Block b finishes sum b of the list.
+__global__ void red_final_kernel(const double* red, const SumList list, double* scal)
 {
     __shared__ double sh[kRedThreads / 32];
+    const double* parts = red + list.at[blockIdx.x];
     // fixed assignment of partials to threads, then a fixed tree: deterministic
     double s = 0.0;
-    for (int i = threadIdx.x; i < count; i += blockDim.x) s += parts[i];
+    for (int i = threadIdx.x; i < list.count[blockIdx.x]; i += blockDim.x) s += parts[i];
     s = block_sum(s, sh);
-    if (threadIdx.x == 0) *out = s;
-}
-
-// parts[b] = this block's sum of d^2, parts[gridDim.x + b] = its sum of c^2
-__global__ void red_pair_kernel(const float* d, const float* c,
-                                size_t n, double* parts)
-{
-    __shared__ double sh[kRedThreads / 32];
-    grid_dependency();
-    // a thread's few terms in FP32 (the ratio only steers the resync
-    // schedule; FP64 arithmetic per element took 46 us on the large volume),
-    // the block's sum in FP64
-    float fd = 0.f, fc = 0.f;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const float a = d[i], b = c[i];
-        fd = fmaf(a, a, fd);
-        fc = fmaf(b, b, fc);
-    }
-    double sd = fd, sc = fc;
-    sd = block_sum(sd, sh);
-    __syncthreads();  // sh is reused
-    sc = block_sum(sc, sh);
-    if (threadIdx.x == 0) {
-        parts[blockIdx.x] = sd;
-        parts[gridDim.x + blockIdx.x] = sc;
-    }
+    if (threadIdx.x == 0) scal[list.slot[blockIdx.x]] = s;
 }
 
 // The refined solve's device-side resync decision for the iteration just
 // finished (sched[1] of them so far): rho = ||d|| / ||c|| joins the budget
 // accumulator; the gate opens (sched[0] = 1) on every R-th iteration or once
 // the accumulated rho exceeds the budget, and the accumulator restarts.
-__global__ void refine_decide_kernel(const double* parts, int count, double* scal, int slot,
-                                     int* sched, int* rlog, int R, double budget)
+// parts[b] = block b's sum of d^2, parts[gridDim.x + b] = its sum of c^2; the
+// last block to arrive (sched[3] counts) adds them in block order and decides.
+// A thread's few terms are summed in FP32 (the ratio only steers the schedule),
+// the blocks' in FP64, which is scarce: 1024 blocks of FP64 tree sums took 10 us
+// on any volume and a second kernel 7 us; 152 blocks and this one take 5 us.
+__global__ void __launch_bounds__(kRedThreads) refine_decide_kernel(const float* d, const float* c,
+                                                                    size_t n, double* parts,
+                                                                    double* scal, int slot,
+                                                                    int* sched, int* rlog, int R,
+                                                                    double budget)
 {
     __shared__ double sh[kRedThreads / 32];
+    __shared__ int s_last;
     grid_dependency();
-    double sd = 0.0, sc = 0.0;
-    for (int i = threadIdx.x; i < count; i += blockDim.x) {
-        sd += parts[i];
-        sc += parts[count + i];
+    float fd[4] = {0.f, 0.f, 0.f, 0.f}, fc[4] = {0.f, 0.f, 0.f, 0.f};
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    const float4* d4 = reinterpret_cast<const float4*>(d);
+    const float4* c4 = reinterpret_cast<const float4*>(c);
+#pragma unroll 4
+    for (size_t i = first; i < n / 4; i += stride) {
+        const float4 a = d4[i], b = c4[i];
+        fd[0] = fmaf(a.x, a.x, fd[0]);
+        fd[1] = fmaf(a.y, a.y, fd[1]);
+        fd[2] = fmaf(a.z, a.z, fd[2]);
+        fd[3] = fmaf(a.w, a.w, fd[3]);
+        fc[0] = fmaf(b.x, b.x, fc[0]);
+        fc[1] = fmaf(b.y, b.y, fc[1]);
+        fc[2] = fmaf(b.z, b.z, fc[2]);
+        fc[3] = fmaf(b.w, b.w, fc[3]);
+    }
+    for (size_t i = n / 4 * 4 + first; i < n; i += stride) {
+        fd[0] = fmaf(d[i], d[i], fd[0]);
+        fc[0] = fmaf(c[i], c[i], fc[0]);
+    }
+    double sd = (double)((fd[0] + fd[1]) + (fd[2] + fd[3]));
+    double sc = (double)((fc[0] + fc[1]) + (fc[2] + fc[3]));
+    sd = block_sum(sd, sh);
+    __syncthreads();  // sh is reused
+    sc = block_sum(sc, sh);
+    if (threadIdx.x == 0) {
+        parts[blockIdx.x] = sd;
+        parts[gridDim.x + blockIdx.x] = sc;
+        __threadfence();
+        s_last = atomicAdd(&sched[3], 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    sd = sc = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+        sd += __ldcg(parts + i);
+        sc += __ldcg(parts + gridDim.x + i);
     }
     sd = block_sum(sd, sh);
     __syncthreads();
@@ -978,6 +997,7 @@ __global__ void refine_decide_kernel(const double* parts, int count, double* sca
     scal[slot] = acc;
     sched[0] = exact;
     sched[1] = it + 1;
+    sched[3] = 0;
     rlog[it & (kRefineLog - 1)] = exact;
 }
 
@@ -1236,11 +1256,79 @@ swopt_status fista_reset_scalars(swopt_handle* h, cudaStream_t st)
     return SWOPT_OK;
 }
 
-static swopt_status finish_reduction(swopt_handle* h, int count, int slot, cudaStream_t st)
+// Room for `count` partial sums of the next entry of the list.
+static double* sum_parts(swopt_handle* h, SumList* list, int count, int slot)
 {
-    red_final_kernel<<<1, kRedThreads, 0, st>>>(h->red, count, h->scal + slot);
+    double* p = h->red + list->used;
+    list->at[list->n] = list->used;
+    list->count[list->n] = count;
+    list->slot[list->n] = slot;
+    ++list->n;
+    list->used += count;
+    return p;
+}
+
+swopt_status finish_sums(swopt_handle* h, const SumList& list, cudaStream_t st)
+{
+    red_final_kernel<<<list.n, kRedThreads, 0, st>>>(h->red, list, h->scal);
     SW_LAUNCHED(h);
     return SWOPT_OK;
+}
+
+swopt_status sum_dot(swopt_handle* h, const float* x, const float* y, size_t n, int slot,
+                     SumList* list, cudaStream_t st)
+{
+    // whole warps of 16-element groups (512 entries)
+    const bool vec = (((uintptr_t)x | (uintptr_t)y) & 15u) == 0;
+    red_dot_kernel<<<kSumBlocks, kRedThreads, 0, st>>>(x, y, n, vec ? n / 512 * 32 : 0,
+                                                       sum_parts(h, list, kSumBlocks, slot));
+    SW_LAUNCHED(h);
+    return SWOPT_OK;
+}
+
+swopt_status sum_states(swopt_handle* h, const float* u, int slot, SumList* list, cudaStream_t st)
+{
+    const int bx = std::max(1, kSumBlocks / h->Q);
+    red_states_kernel<<<dim3(bx, h->Q), kRedThreads, 0, st>>>(u, (size_t)h->S * h->Twp, h->Cmf,
+                                                              sum_parts(h, list, bx * h->Q, slot));
+    SW_LAUNCHED(h);
+    return SWOPT_OK;
+}
+
+swopt_status sum_abs(swopt_handle* h, const float* x, size_t n, int slot, SumList* list,
+                     cudaStream_t st)
+{
+    red_abs_kernel<<<kSumBlocks, kRedThreads, 0, st>>>(x, n, sum_parts(h, list, kSumBlocks, slot));
+    SW_LAUNCHED(h);
+    return SWOPT_OK;
+}
+
+swopt_status sum_tv(swopt_handle* h, const float* x, int slot, SumList* list, cudaStream_t st)
+{
+    red_tv_kernel<<<kSumBlocks, kRedThreads, 0, st>>>(x, vol_of(h),
+                                                      sum_parts(h, list, kSumBlocks, slot));
+    SW_LAUNCHED(h);
+    return SWOPT_OK;
+}
+
+swopt_status sum_tv_states(swopt_handle* h, const float* b, int slot, SumList* list,
+                           cudaStream_t st)
+{
+    Vol v = vol_of(h);
+    v.P = h->Q;
+    v.L = nb_of(h);
+    red_tv_weighted_kernel<<<kSumBlocks, kRedThreads, 0, st>>>(
+        b, v, h->Cmf, sum_parts(h, list, kSumBlocks, slot));
+    SW_LAUNCHED(h);
+    return SWOPT_OK;
+}
+
+swopt_status reduce_dot(swopt_handle* h, const float* x, const float* y, size_t n, int slot,
+                        cudaStream_t st)
+{
+    SumList list;
+    SW_TRY(sum_dot(h, x, y, n, slot, &list, st));
+    return finish_sums(h, list, st);
 }
 
 swopt_status reduce_sumsq(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st)
@@ -1248,64 +1336,14 @@ swopt_status reduce_sumsq(swopt_handle* h, const float* x, size_t n, int slot, c
     return reduce_dot(h, x, x, n, slot, st);
 }
 
-swopt_status reduce_dot(swopt_handle* h, const float* x, const float* y, size_t n, int slot,
-                        cudaStream_t st)
-{
-    // whole warps of 16-element groups (512 entries)
-    const bool vec = (((uintptr_t)x | (uintptr_t)y) & 15u) == 0;
-    red_dot_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(x, y, n, vec ? n / 512 * 32 : 0, h->red);
-    SW_LAUNCHED(h);
-    return finish_reduction(h, kRedBlocks, slot, st);
-}
-
-swopt_status reduce_states(swopt_handle* h, const float* u, int slot, cudaStream_t st)
-{
-    const int bx = std::max(1, kRedBlocks / h->Q);
-    red_states_kernel<<<dim3(bx, h->Q), kRedThreads, 0, st>>>(u, (size_t)h->S * h->Twp, h->Cmf,
-                                                              h->red);
-    SW_LAUNCHED(h);
-    return finish_reduction(h, bx * h->Q, slot, st);
-}
-
-swopt_status reduce_abs(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st)
-{
-    red_abs_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(x, n, h->red);
-    SW_LAUNCHED(h);
-    return finish_reduction(h, kRedBlocks, slot, st);
-}
-
-swopt_status reduce_tv(swopt_handle* h, const float* x, int slot, cudaStream_t st)
-{
-    red_tv_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(x, vol_of(h), h->red);
-    SW_LAUNCHED(h);
-    return finish_reduction(h, kRedBlocks, slot, st);
-}
-
-swopt_status reduce_tv_states(swopt_handle* h, const float* b, int slot, cudaStream_t st)
-{
-    Vol v = vol_of(h);
-    v.P = h->Q;
-    v.L = nb_of(h);
-    red_tv_weighted_kernel<<<kRedBlocks, kRedThreads, 0, st>>>(b, v, h->Cmf, h->red);
-    SW_LAUNCHED(h);
-    return finish_reduction(h, kRedBlocks, slot, st);
-}
-
-swopt_status reduce_partials(swopt_handle* h, const double* parts, int count, int slot,
-                             cudaStream_t st)
-{
-    red_final_kernel<<<1, kRedThreads, 0, st>>>(parts, count, h->scal + slot);
-    SW_LAUNCHED(h);
-    return SWOPT_OK;
-}
-
 swopt_status refine_decide(swopt_handle* h, const float* d, const float* c, int slot, int R,
                            double budget, cudaStream_t st)
 {
-    SW_CUDA(launch_pdl(red_pair_kernel, kRedBlocks, kRedThreads, 0, st, d, c, nc_of(h), h->red));
-    SW_LAUNCHED(h);
-    SW_CUDA(launch_pdl(refine_decide_kernel, 1, kRedThreads, 0, st, h->red, kRedBlocks, h->scal, slot,
-                       h->sched, h->rlog, R, budget));
+    // eight 16-byte pairs per thread at most one block per SM, more terms beyond
+    const size_t n = nc_of(h);
+    const int grid = std::max(1, std::min(grid_for(n, kRedThreads * 16), 152));
+    SW_CUDA(launch_pdl(refine_decide_kernel, grid, kRedThreads, 0, st, d, c, n, h->red, h->scal,
+                       slot, h->sched, h->rlog, R, budget));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }

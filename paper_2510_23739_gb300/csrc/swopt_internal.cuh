@@ -362,7 +362,7 @@ swopt_status fft_forward(swopt_handle* h, const float* c, const float* ytil, int
 // 2 as launch_pt_refine.
 struct FftImage {
     bool per_state = false;
-    int mode = 0, add = 0;
+    int mode = 0, add = 0, add2 = 0;
     float alpha = 0.f;
     float* out = nullptr;
     const float* xi = nullptr;
@@ -379,6 +379,14 @@ swopt_status fft_adjoint(swopt_handle* h, const float* src, bool from_y, bool ro
 enum class FftKeep { never, always, nonfinite };
 swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool round, FftKeep keep,
                         const FftImage& img, cudaStream_t st);
+// The refined solve's step decided on the device, in one chain of launches: by
+// h->sched[0], 0: G += H^T H delta with operands rounded if `round`; else
+// G = H^T (H c - ytil), rounded if `round2`; the rest as launch_pt_refine
+// (img.mode 2).  Only where fft_refine_gated (one tile), and not with round2
+// alone.
+bool fft_refine_gated(const swopt_handle* h);
+swopt_status fft_refine(swopt_handle* h, const float* delta, const float* c, const float* ytil,
+                        bool round, bool round2, const FftImage& img, cudaStream_t st);
 // Multiply-adds of the spectral product of A (0) or A^T (1)
 double fft_issued_macs(const swopt_handle* h, int kernel);
 
@@ -436,14 +444,26 @@ swopt_status fista_reset_scalars(swopt_handle* h, cudaStream_t st);
 swopt_status reduce_sumsq(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st);
 swopt_status reduce_dot(swopt_handle* h, const float* x, const float* y, size_t n, int slot,
                         cudaStream_t st);
-// sum_m Cm[m] ||u_m||^2 of u [Q][Y][X][Twp]
-swopt_status reduce_states(swopt_handle* h, const float* u, int slot, cudaStream_t st);
-swopt_status reduce_abs(swopt_handle* h, const float* x, size_t n, int slot, cudaStream_t st);
-swopt_status reduce_tv(swopt_handle* h, const float* x, int slot, cudaStream_t st);
+// Several sums finished by one kernel: each sum_* launches its first pass into
+// its own part of h->red, finish_sums writes every result to its slot of h->scal.
+// sum_states (up to 4096 partial sums) comes last.
+constexpr int kSumBlocks = 608;  // blocks of a first pass: four per SM
+constexpr int kObjectiveSums = 4 * kSumBlocks + 4096;
+struct SumList {
+    int n = 0, used = 0;
+    int at[8], count[8], slot[8];
+};
+swopt_status sum_dot(swopt_handle* h, const float* x, const float* y, size_t n, int slot,
+                     SumList* list, cudaStream_t st);
+swopt_status sum_abs(swopt_handle* h, const float* x, size_t n, int slot, SumList* list,
+                     cudaStream_t st);
+swopt_status sum_tv(swopt_handle* h, const float* x, int slot, SumList* list, cudaStream_t st);
 // sum_m Cm[m] TV(b_m) of the Q state images b [Q][Y][X][Z] (= sum_n TV((S c)^n))
-swopt_status reduce_tv_states(swopt_handle* h, const float* b, int slot, cudaStream_t st);
-swopt_status reduce_partials(swopt_handle* h, const double* parts, int count, int slot,
-                             cudaStream_t st);
+swopt_status sum_tv_states(swopt_handle* h, const float* b, int slot, SumList* list,
+                           cudaStream_t st);
+// sum_m Cm[m] ||u_m||^2 of u [Q][Y][X][Twp]
+swopt_status sum_states(swopt_handle* h, const float* u, int slot, SumList* list, cudaStream_t st);
+swopt_status finish_sums(swopt_handle* h, const SumList& list, cudaStream_t st);
 // Refined solve, device-side schedule: rho = ||d|| / ||c|| (FP64) is added
 // to the budget accumulator scal[slot]; the gate h->sched[0] opens the exact
 // resync when the iteration is a multiple of R or the accumulated sum

@@ -47,6 +47,46 @@ def test_solves_of_one_handle_equal_those_of_fresh_handles(prec, kw):
         one.close()
 
 
+@pytest.mark.parametrize("prec", ["fp32", "bf16x3", "bf16"])
+@pytest.mark.parametrize("resync", ["fp32", "bf16x3", "bf16"])
+@pytest.mark.parametrize("budget", [0.0, 0.05])
+def test_resync_precisions(prec, resync, budget):
+    """Every pair of increment and resync precisions, decided on the host or
+    on the device: the plain FP32 iterates to BF16's operator error (5e-3)."""
+    op = sw.Operator(GEOM, K, SW)
+    try:
+        want = _solve(op, _y(6), _params())
+        op.set_precision(prec)
+        got = _solve(op, _y(6), _params(refine_every=2, refine_precision=resync,
+                                        refine_budget=budget))
+        op.check_device()
+        assert float((got - want).norm() / want.norm()) <= 5e-3
+        if "bf16" not in (prec, resync):
+            assert float((got - want).norm() / want.norm()) <= 1e-5
+    finally:
+        op.close()
+
+
+def test_unpinning_a_tensor_core_schedule():
+    """A schedule pinned before the precision is selected, then released."""
+    op = sw.Operator(GEOM, K, SW)
+    try:
+        for kid in (0, 1):
+            op.tc_schedule(kid, split=1)
+        op.set_precision("bf16")
+        c = torch.tensor(np.random.default_rng(7).standard_normal(GEOM.c_shape()),
+                         dtype=torch.float32, device="cuda")
+        pinned = op.forward(c), op.adjoint(_y(8))
+        for kid in (0, 1):
+            op.tc_schedule(kid)
+        free = op.forward(c), op.adjoint(_y(8))
+        op.check_device()
+        for a, b in zip(pinned, free):
+            assert float((a - b).norm() / b.norm()) <= 2e-5  # FP32 sums of the same products
+    finally:
+        op.close()
+
+
 def test_a_restored_step_is_not_taken_for_the_next_solve():
     a, b = sw.Operator(GEOM, K, SW), sw.Operator(GEOM, K, SW)
     try:
