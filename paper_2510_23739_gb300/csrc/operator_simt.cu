@@ -270,34 +270,36 @@ __global__ void states_kernel(const float* __restrict__ c, const float* __restri
 }
 
 // y[n][s][t] = u[n mod ncyc][s][t - t0] inside the window, 0 outside.  Bound by
-// the stores of y: a warp writes whole rows (n, s), VEC floats per lane and
-// store (4 where T is a multiple of 4 and y 16-byte aligned: t0 is a multiple
-// of 4), with streaming stores, since y is far larger than L2.  20 x 128^2 x 320
-// floats (0.42 GB): 85 us; 289 us with 64-bit divisions per element and 4-byte
-// stores.
+// the stores of y: a warp takes a row (m, s) of u, reads it once and writes the
+// rows of all pulses of state m, VEC floats per lane and store (4 where T is a
+// multiple of 4 and y 16-byte aligned: t0 is a multiple of 4), with streaming
+// stores, since y is far larger than L2.
 template <int VEC>
-__global__ void expand_kernel(const float* u, float* y, int N, int S,
-                              int T, int ncyc, int t0, int Twp)
+__global__ void expand_kernel(const float* u, float* y, int N, int Q, int S, int T, int ncyc,
+                              int t0, int Twp)
 {
     grid_dependency();
     const int lane = threadIdx.x & 31;
     const unsigned warps = gridDim.x * (blockDim.x >> 5);
+    const size_t step = (size_t)ncyc * S * T;
     for (size_t row = blockIdx.x * (size_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-         row < (size_t)N * S; row += warps) {
-        const int n = (int)(row / (unsigned)S);
-        const float* src = u + ((size_t)(n % ncyc) * S + (row - (size_t)n * S)) * Twp;
-        float* dst = y + row * T;
-        if (VEC == 4) {
-            for (int t = 4 * lane; t < T; t += 128) {
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                const int w = t - t0;
-                if (w >= 0 && w < Twp) v = load_produced(reinterpret_cast<const float4*>(src + w));
-                __stcs(reinterpret_cast<float4*>(dst + t), v);
-            }
-        } else {
-            for (int t = lane; t < T; t += 32) {
-                const int w = t - t0;
-                __stcs(dst + t, w >= 0 && w < Twp ? load_produced(src + w) : 0.f);
+         row < (size_t)Q * S; row += warps) {
+        const int m = (int)(row / (unsigned)S);
+        const float* src = u + row * Twp;
+        float* dst = y + ((size_t)m * S + (row - (size_t)m * S)) * T;
+        for (int t = VEC * lane; t < T; t += 32 * VEC) {
+            const int w = t - t0;
+            const bool in = w >= 0 && w < Twp;
+            float* p = dst + t;
+            if (VEC == 4) {
+                const float4 v = in ? load_produced(reinterpret_cast<const float4*>(src + w))
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+                for (int n = m; n < N; n += ncyc, p += step) __stcs(reinterpret_cast<float4*>(p), v);
+            } else {
+                const float v = in ? load_produced(src + w) : 0.f;
+#pragma unroll 4
+                for (int n = m; n < N; n += ncyc, p += step) __stcs(p, v);
             }
         }
     }
@@ -474,10 +476,10 @@ swopt_status launch_states(swopt_handle* h, const float* c, float* b, cudaStream
 
 swopt_status launch_expand(swopt_handle* h, const float* u, float* y, cudaStream_t st)
 {
-    const int grid = std::min(grid_for((size_t)h->N * h->S, 8), 152 * 16);
+    const int grid = std::min(grid_for((size_t)h->Q * h->S, 8), 152 * 8);
     const bool vec = h->T % 4 == 0 && ((uintptr_t)y & 15u) == 0;
     SW_CUDA(launch_pdl(vec ? expand_kernel<4> : expand_kernel<1>, grid, 256, 0, st, u, y, h->N,
-                       h->S, h->T, h->ncyc, h->t0, h->Twp));
+                       h->Q, h->S, h->T, h->ncyc, h->t0, h->Twp));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
