@@ -932,7 +932,8 @@ __global__ void red_final_kernel(const double* red, const SumList list, double* 
 // last block to arrive (sched[3] counts) adds them in block order and decides.
 // A thread's few terms are summed in FP32 (the ratio only steers the schedule),
 // the blocks' in FP64, which is scarce: 1024 blocks of FP64 tree sums took 10 us
-// on any volume and a second kernel 7 us; 152 blocks and this one take 5 us.
+// on any volume and a second kernel 7 us; this one takes 5 us on small volumes and
+// 17 us on 3 x 128^2 x 96 (152 blocks there left too few loads in flight: 25 us).
 __global__ void __launch_bounds__(kRedThreads) refine_decide_kernel(const float* d, const float* c,
                                                                     size_t n, double* parts,
                                                                     double* scal, int slot,
@@ -1056,14 +1057,19 @@ __global__ void __launch_bounds__(128) param_partial_kernel(const float* __restr
     }
 }
 
+// W[i] = sum over the chunks, a warp per output: lane l adds chunks l, l + 32, ...,
+// then a tree (one thread per output chained 110 FP64 additions: 15 us; now 5).
 __global__ void param_final_kernel(const double* __restrict__ parts, double* __restrict__ W, int n,
                                    int chunks)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int k = 0; k < chunks; ++k) s += parts[(size_t)k * n + i];
-        W[i] = s;
-    }
+    const int lane = threadIdx.x & 31;
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (i >= n) return;
+    double s = 0.0;
+    for (int k = lane; k < chunks; k += 32) s += parts[(size_t)k * n + i];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) W[i] = s;
 }
 
 Vol vol_of(const swopt_handle* h)
@@ -1339,9 +1345,9 @@ swopt_status reduce_sumsq(swopt_handle* h, const float* x, size_t n, int slot, c
 swopt_status refine_decide(swopt_handle* h, const float* d, const float* c, int slot, int R,
                            double budget, cudaStream_t st)
 {
-    // eight 16-byte pairs per thread at most one block per SM, more terms beyond
+    // four 16-byte pairs per thread, up to four blocks per SM, more terms beyond
     const size_t n = nc_of(h);
-    const int grid = std::max(1, std::min(grid_for(n, kRedThreads * 16), 152));
+    const int grid = std::max(1, std::min(grid_for(n, kRedThreads * 16), kSumBlocks));
     SW_CUDA(launch_pdl(refine_decide_kernel, grid, kRedThreads, 0, st, d, c, n, h->red, h->scal,
                        slot, h->sched, h->rlog, R, budget));
     SW_LAUNCHED(h);
@@ -1375,7 +1381,7 @@ swopt_status param_weights(swopt_handle* h, const float* g, const float* c, int 
     param_partial_kernel<<<dim3(chunks, h->Q, (h->P + 3) / 4), 128, 0, st>>>(
         g, c, h->pparts, h->Q, h->P, h->S, h->Z, run);
     SW_LAUNCHED(h);
-    param_final_kernel<<<(n + 127) / 128, 128, 0, st>>>(h->pparts, h->red + slot0, n, chunks);
+    param_final_kernel<<<(n + 3) / 4, 128, 0, st>>>(h->pparts, h->red + slot0, n, chunks);
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
