@@ -287,7 +287,17 @@ bool use_tc(const swopt_handle* h) { return h->precision != SWOPT_PREC_FP32; }
 
 // True when the spectral kernels serve the handle's precision: every one but
 // FP8, unless a tensor-core tiling or schedule is pinned (swopt_tc_configure,
-// swopt_tc_schedule), which asks for those kernels.
+// swopt_tc_schedule), which asks for those kernels.  No line by support or size:
+// one FISTA iteration without TV, us, direct kernels / spectral ones, 10 states:
+//                      k = 1         k = 3         k = 7         k = 11
+//   16^2 x 24   FP32   88 / 50      218 / 50      895 / 50     2767 / 52
+//               BF16  122 / 50      125 / 50      142 / 52      177 / 54
+//   64^2 x 64   FP32  187 / 92      438 / 129    1709 / 129    4581 / 135
+//               BF16  269 / 105     281 / 142     326 / 142     394 / 148
+//   128^2 x 96  FP32  989 / 417   2296 / 477    8864 / 503   22842 / 466
+//               BF16  758 / 464    801 / 540     932 / 558    1156 / 510
+// and with 1 state, BF16, 128^2 x 96: 241 / 192 (k = 1), 250 / 163, 298 / 186.
+// The least gain found is k = 1 in FP32 with 1 state on 320 x 300: 356 / 346.
 bool route_fft(const swopt_handle* h)
 {
     if (!h->fft || h->precision == SWOPT_PREC_FP8) return false;

@@ -8,9 +8,10 @@
 //   u^_m[t](f) = sum_j K^[j][t](f) b^_m[j](f),   b^_m = sum_p S[m][p] c^_p,
 // exact in real arithmetic.  The direct sums of the largest workload are 741
 // GFLOP (31 x 31 taps); here they are 4 GFLOP of products and 1 GFLOP of
-// transforms, so every kernel of this file is bound by memory, and the
-// operator runs in FP32 throughout (error 3e-7 to 5e-7 against 64 bits where
-// the direct FP32 sums, chains of 10^4 products, have 7e-7 to 5e-6).
+// transforms, in FP32 throughout (error 1e-7 to 2e-7 against 64 bits where the
+// direct FP32 sums, chains of 10^4 products, have 4e-7 to 5e-6).  H^T H of that
+// workload: 0.60 ms; the direct sums took 130 + 130 ms on the CUDA cores and, in
+// BF16 on the tensor cores at 98% of their peak over the padded band, 2.2 + 2.4 ms.
 //
 // Structure used:
 //  * Two neighbouring channels (depths or samples) are the real and imaginary
@@ -387,8 +388,11 @@ __device__ __noinline__ float direct_adjoint(const FftShape& s, int round, const
 
 // ---------------------------------------------------------------------------
 // Transforms along x and y.  A block takes 32 lines, one per lane: neighbouring
-// lanes are neighbouring channel pairs (then rows, or x frequencies).  Bound by
-// memory: a pass reads and writes every value once.
+// lanes are neighbouring channel pairs (then rows, or x frequencies).  A pass
+// reads and writes every value once and is bound by memory and its latency: at
+// three blocks per SM (80 registers; with two 10 to 20% slower) the y pass moves
+// 10 x 144^2 x 56 pairs, 186 MB, in 29 us, 6.4 TB/s (mostly L2), and the x passes,
+// whose sources are strided, 160 MB in 49 to 54 us.
 // ---------------------------------------------------------------------------
 // SRC_GATED: SRC_STATES, or SRC_C as the second variant
 enum { SRC_C = 0, SRC_STATES = 1, SRC_U = 2, SRC_Y = 3, SRC_GATED = 4 };
@@ -912,8 +916,11 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
 // ring of asynchronous copies that runs ahead across the warp's groups and
 // starts before the inputs are staged; a thread reads back only what it copied
 // itself, so the ring needs no barrier.
-// Bound by the K^ stream (HBM) for few states, by the FMA rate from about 10
-// states on.
+// Bound by latency and shared-memory reads at 14 to 16 warps per SM (the inputs
+// of 10 states take 61 KB per block): 145 us per product of the largest workload
+// (k = 31, 10 states), where the K^ stream alone is 56 us of HBM time and the FMAs
+// 48 us.  One register accumulator per value with K^ read by the thread itself:
+// 200 us (164 to 255 registers, one block per SM).
 // ---------------------------------------------------------------------------
 struct Spec {
     FftShape s;
@@ -949,8 +956,11 @@ __device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b)
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
-constexpr int kRingRows = 4;    // contracted channels per ring slot
-constexpr int kRingSlots = 3;   // two in flight while one is consumed
+// Contracted channels per ring slot, and slots (two in flight while one is consumed).
+// 2 x 4 gave 1% on 128^2 planes, but 53 for 44 us on 45 x 37, where a block has its
+// SM to itself and the waits per row count; 2 x 6, 1 x 8 and 8 x 2 are slower on all.
+constexpr int kRingRows = 4;
+constexpr int kRingSlots = 3;
 
 // float2 slots per (channel, frequency) of the staged inputs: MC, padded so
 // that 8 frequencies start in 8 different 16-byte bank groups
@@ -1523,7 +1533,10 @@ void fft_prepare(swopt_handle* h)
 
     // lengths: the least estimated time over all pairs (K^ and the spectra through
     // memory at 5 TB/s, the products at 40 TFLOP/s), for a nominal number of
-    // states: shards of one problem take the same lengths, hence the same bits
+    // states: shards of one problem take the same lengths, hence the same bits.
+    // The tiles of a k = 1 kernel do not overlap, so that small ones cost the same in
+    // this estimate: few are preferred (one H^T H at 128^2 x 96 in 4 x 4 tiles 717 us,
+    // in one 417; 64^2 x 64 139 and 92)
     const double states = 8.0;
     double best = 1e300;
     FftAxis by{}, bx{};
@@ -1538,7 +1551,8 @@ void fft_prepare(swopt_handle* h)
             const double work = 8.0 * tiles * area * std::max(h->Q * Ct2, h->Q * Cz2);
             // memory limits: 24 GB of K^ (twice with the BF16 one), 8 GB per workspace
             if (kbytes > 24e9 || work > 8e9) continue;
-            const double t = std::max(kbytes / 5e12, flops / 40e12) + sbytes / 5e12;
+            double t = std::max(kbytes / 5e12, flops / 40e12) + sbytes / 5e12;
+            if (h->r == 0) t *= 1.0 + 0.02 * tiles;
             if (t < best) {
                 best = t;
                 by = y;

@@ -188,3 +188,17 @@ def test_solve_with_a_nan_measurement_keeps_the_rest():
         assert float((got - whole)[:, ~near].norm() / whole[:, ~near].norm()) <= 1e-5
     finally:
         op.close()
+
+
+@pytest.mark.parametrize("X,Y", [(16, 18), (11, 258), (257, 5)])
+def test_one_tap(X, Y):
+    """k = 1: tiles that do not overlap, one where the scan fits, else several."""
+    g, s, K = problem(X=X, Y=Y, Z=5, T=12, N=3, P=2, k=1, cycle=2)
+    rng = np.random.default_rng(9)
+    c, y = rng.standard_normal(g.c_shape()), rng.standard_normal(g.y_shape())
+    op = sw.Operator(g, K, s)
+    try:
+        assert rel(host(op.forward(dev(c))), oracle.forward(g, s, K, c)) <= TOL
+        assert rel(host(op.adjoint(dev(y))), oracle.adjoint(g, s, K, y)) <= TOL
+    finally:
+        op.close()
