@@ -483,7 +483,8 @@ swopt_status swopt_check_device(swopt_handle* h, void* stream);
 /* FLOPs issued by one launch of the A (kernel_id 0) or A^T (1) contraction in
  * the current precision: 2 x the multiply-adds the kernel executes,
  * including the zero-padded parts of the kernel band it does not skip (for
- * the split BF16 modes, all 3 or 6 products). */
+ * the split BF16 modes on the tensor cores, all 3 or 6 products; by FFTs those
+ * of the product of the spectra, without the transforms). */
 swopt_status swopt_issued_flops(swopt_handle* h, int kernel_id, double* flops);
 
 /* Tensor-core tile configuration (autotuner).  When a BF16 precision is
