@@ -466,9 +466,9 @@ def run_prox_joint(args, device):
     """The prox of the full R3 with its lambda_3 term (swopt_prox_joint) on
     the workload's volume and switching states: time per call of `inner` dual
     iterations, CUDA events over `steps` calls after `warmup`.  Per dual
-    iteration (one dual per switching state, nd = 4 P + 3 Q volumes): L^T
-    reads the momentum duals and z and writes w (nd + 2 P volumes); the update
-    reads w, reads and writes u and r (4 nd + P volumes).  The duals of the
+    iteration (one dual per switching state, nd = 4 P + 3 Q volumes): w from
+    the sums for L^T and z (6 P volumes); the dual step reads w and two dual
+    iterates and writes one and the sums (3 nd + 5 P volumes).  The duals of the
     large workload (P = 3, Q = 10) are 42 volumes of 6.3 MB, twice L2 per
     array."""
     import torch
@@ -505,7 +505,7 @@ def run_prox_joint(args, device):
     ms = e0.elapsed_time(e1) / args.steps
     L = g.Y * g.X * g.Z
     nd = 4 * g.P + 3 * states
-    bytes_iter = 4.0 * L * ((nd + 2 * g.P) + (4 * nd + g.P))
+    bytes_iter = 4.0 * L * (3 * nd + 11 * g.P)
     gbs = bytes_iter * inner / (ms * 1e-3) / 1e9
     peaks, src = _peaks()
     print(json.dumps({
@@ -573,7 +573,7 @@ def run_prox_tv(args, device):
                    "l2": "dual arrays 3 x 19 MB per component block, 190 MB in all (no flush)"},
         "roofline": {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": gbs / peaks["hbm_gbs"], "traffic": None,
-                     "moved_gb_per_s": 72.0 * n * inner / (ms * 1e-3) / 1e9,
+                     "note": "volumes that fit stay on the chip between inner iterations",
                      "peak_source": f"HBM copy ({src})"},
         "clocks": clk}), flush=True)
 
