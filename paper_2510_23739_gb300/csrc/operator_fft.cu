@@ -1638,16 +1638,17 @@ FftShape shape_of(const swopt_handle* h, bool round)
 
 bool aligned8(const void* p) { return ((uintptr_t)p & 7u) == 0; }
 
-// Launches a line-transform kernel over `items` lines along axis `ax`.
+// Launches a line-transform kernel over `items` lines along axis `ax` (the larger
+// count where the device picks between two variants).
 template <class Args>
-swopt_status launch_lines(swopt_handle* h, void (*kernel)(const Args), const Args& a,
+swopt_status launch_lines(swopt_handle* h, void (*kernel)(const Args), const Args& a, unsigned items,
                           const FftAxis& ax, cudaStream_t st)
 {
     const size_t smem = (size_t)ax.L * 32 * sizeof(float2);
     if (smem > 48 * 1024)
         SW_CUDA(cudaFuncSetAttribute((const void*)kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    SW_CUDA(launch_pdl(kernel, (a.items + 31) / 32, 32 * fft_warps(ax), smem, st, a));
+    SW_CUDA(launch_pdl(kernel, (items + 31) / 32, 32 * fft_warps(ax), smem, st, a));
     SW_LAUNCHED(h);
     return SWOPT_OK;
 }
@@ -1662,7 +1663,8 @@ swopt_status launch_y(swopt_handle* h, const FftShape& s, bool inverse, int plan
     a.width = (unsigned)(s.x.L * C2);
     a.items = (unsigned)(planes * s.tiles) * a.width;
     a.items2 = (unsigned)(planes2 * s.tiles) * a.width;
-    return launch_lines(h, inverse ? fft_y_kernel<1> : fft_y_kernel<-1>, a, s.y, st);
+    return launch_lines(h, inverse ? fft_y_kernel<1> : fft_y_kernel<-1>, a,
+                        std::max(a.items, a.items2), s.y, st);
 }
 
 template <int MC, bool ADJ, int MAP>
@@ -1740,7 +1742,7 @@ swopt_status forward_to_lines(swopt_handle* h, const FftShape& s, const float* c
                         gated     ? fft_x_forward_kernel<SRC_GATED>
                         : s.round ? fft_x_forward_kernel<SRC_STATES>
                                   : fft_x_forward_kernel<SRC_C>,
-                        a, f->x, st));
+                        a, std::max(a.items, a.items2), f->x, st));
     SW_TRY(launch_y(h, s, false, planes, planes2, f->Cz2, f->w0, f->w1, st));
     if (gated) SW_TRY((launch_spec<false, MAP_GATED>(h, s, f->w1, f->w0, st)));
     else if (s.round) SW_TRY((launch_spec<false, MAP_NONE>(h, s, f->w1, f->w0, st)));
@@ -1781,7 +1783,7 @@ swopt_status adjoint_from_lines(swopt_handle* h, const FftShape& s, const float*
                         img.mode == IMG_STORE  ? fft_x_image_kernel<IMG_STORE>
                         : img.mode == IMG_STEP ? fft_x_image_kernel<IMG_STEP>
                                                : fft_x_image_kernel<IMG_REFINE>,
-                        v, f->x, st);
+                        v, v.items, f->x, st);
 }
 
 }  // namespace
@@ -1804,7 +1806,7 @@ swopt_status fft_forward(swopt_handle* h, const float* c, const float* ytil, int
     v.ytil = ytil;
     v.Cmf = scale ? h->Cmf : nullptr;
     v.c = c;
-    SW_TRY(launch_lines(h, fft_x_u_kernel, v, f->x, st));
+    SW_TRY(launch_lines(h, fft_x_u_kernel, v, v.items, f->x, st));
     prof_end(h, &rec, st);
     return SWOPT_OK;
 }
@@ -1824,7 +1826,7 @@ swopt_status fft_adjoint(swopt_handle* h, const float* src, bool from_y, bool ro
     ProfileRec rec;
     prof_begin(h, 1, st, &rec);
     SW_TRY(launch_lines(h, from_y ? fft_x_forward_kernel<SRC_Y> : fft_x_forward_kernel<SRC_U>, a,
-                        f->x, st));
+                        a.items, f->x, st));
     SW_TRY(adjoint_from_lines(h, s, src, from_y, KEEP_ALWAYS, KEEP_ALWAYS, img, st));
     prof_end(h, &rec, st);
     return SWOPT_OK;
