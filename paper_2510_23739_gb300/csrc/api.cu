@@ -127,7 +127,7 @@ swopt_status dalloc(T** p, size_t count)
     if (e != cudaSuccess) {
         *p = nullptr;
         set_error("cudaMalloc of %zu bytes failed: %s", count * sizeof(T), cudaGetErrorString(e));
-        return e == cudaErrorMemoryAllocation ? SWOPT_ERR_OOM : SWOPT_ERR_CUDA;
+        return cuda_status(e);
     }
     return SWOPT_OK;
 }

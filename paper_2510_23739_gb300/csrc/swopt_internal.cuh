@@ -17,13 +17,22 @@ namespace swopt {
 void set_error(const char* fmt, ...);
 void clear_error();
 
+// The status of a failed runtime call.  An allocation that failed is reported here
+// and not again by the next launch's check: a caller may free memory and go on.
+inline swopt_status cuda_status(cudaError_t e)
+{
+    if (e != cudaErrorMemoryAllocation) return SWOPT_ERR_CUDA;
+    cudaGetLastError();
+    return SWOPT_ERR_OOM;
+}
+
 #define SW_CUDA(call)                                                              \
     do {                                                                           \
         cudaError_t e_ = (call);                                                   \
         if (e_ != cudaSuccess) {                                                   \
             ::swopt::set_error("%s failed: %s (%s:%d)", #call, cudaGetErrorString(e_), \
                                __FILE__, __LINE__);                                \
-            return e_ == cudaErrorMemoryAllocation ? SWOPT_ERR_OOM : SWOPT_ERR_CUDA; \
+            return ::swopt::cuda_status(e_);                                       \
         }                                                                          \
     } while (0)
 
