@@ -460,14 +460,18 @@ size_t march_smem(int TY, int TX, int V)
 }  // namespace
 
 // Chooses the tile (h->march.TY = -1: the volume does not fit) and allocates the
-// counters.  Synchronous; not while capturing.
+// counters.  The handle's plan is set at the end, when everything it names exists: a
+// call that failed leaves none.  Synchronous; not while capturing.
 swopt_status march_prepare(swopt_handle* h)
 {
-    MarchPlan& m = h->march;
-    if (m.TY != 0) return SWOPT_OK;
+    if (h->march.TY != 0) return SWOPT_OK;
+    MarchPlan m;
     m.TY = -1;
     const int V = (h->Z + 31) / 32;
-    if (V > 4) return SWOPT_OK;
+    if (V > 4) {
+        h->march = m;
+        return SWOPT_OK;
+    }
     int sms = 0, sm_smem = 0;
     SW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
     SW_CUDA(cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device));
@@ -511,7 +515,10 @@ swopt_status march_prepare(swopt_handle* h)
             }
         }
     }
-    if (m.TY < 0) return SWOPT_OK;
+    if (m.TY < 0) {
+        h->march = m;
+        return SWOPT_OK;
+    }
     const MarchKernel k = march_kernel(V, m.TY, m.TX);
     int per_sm = 0;
     SW_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -519,19 +526,26 @@ swopt_status march_prepare(swopt_handle* h)
     SW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * (m.TX + 1),
                                                           march_smem(m.TY, m.TX, V)));
     if ((long)per_sm * sms < m.blocks) {  // the estimate was too high
-        m.TY = -1;
+        h->march = MarchPlan();
+        h->march.TY = -1;
         return SWOPT_OK;
     }
-    if (!m.flags) {
-        SW_CUDA(cudaMalloc((void**)&m.flags, sizeof(unsigned) * m.blocks));
-        SW_CUDA(cudaMemset(m.flags, 0, sizeof(unsigned) * m.blocks));
+    SW_CUDA(cudaMalloc((void**)&m.flags, sizeof(unsigned) * m.blocks));
+    if (cudaError_t e = cudaMemset(m.flags, 0, sizeof(unsigned) * m.blocks); e != cudaSuccess) {
+        cudaFree(m.flags);
+        SW_CUDA(e);
     }
+    h->march = m;
     return SWOPT_OK;
 }
 
 swopt_status march_launch(swopt_handle* h, const MarchCall& call, cudaStream_t st)
 {
     const MarchPlan& m = h->march;
+    if (m.TY <= 0 || !m.flags) {
+        set_error("internal: no plan of the TV prox");
+        return SWOPT_ERR_DEVICE_CHECK;
+    }
     const int V = (h->Z + 31) / 32;
     March a{};
     a.z = call.z;
