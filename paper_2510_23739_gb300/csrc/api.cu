@@ -879,12 +879,15 @@ swopt_status swopt_create(const swopt_geometry* geom, const double* K_host,
 
     swopt_handle* h = new swopt_handle();
     h->X = g.X; h->Y = g.Y; h->Z = g.Z; h->T = g.T; h->N = g.N; h->P = g.P; h->k = g.k;
-    h->r = g.k / 2; h->ncyc = g.pulses_per_cycle; h->dz_mm = g.dz_mm; h->mu = sw->mu_per_mm;
+    h->r = g.k / 2; h->dz_mm = g.dz_mm; h->mu = sw->mu_per_mm;
+    // a cycle past the last pulse is never completed: n mod cycle = n for all of them, and
+    // a count within N keeps n + cycle (the loops over the pulses of a state) in range
+    h->ncyc = std::min(g.N, g.pulses_per_cycle);
     h->kappa.assign(sw->kappa_host, sw->kappa_host + g.P);
     h->eps_bar.assign(sw->eps_bar_host, sw->eps_bar_host + g.P);
     h->eps_off.assign(sw->eps_off_host, sw->eps_off_host + g.P);
     h->S = g.X * g.Y;
-    h->Q = std::min(g.N, g.pulses_per_cycle);
+    h->Q = h->ncyc;
     h->nnz = nnz;
     h->t0 = tmin & ~3;
     h->tw = tmax - h->t0 + 1;
