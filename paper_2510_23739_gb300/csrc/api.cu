@@ -302,6 +302,7 @@ bool route_fft(const swopt_handle* h)
 {
     if (!h->fft || h->precision == SWOPT_PREC_FP8) return false;
     if (h->precision == SWOPT_PREC_FP32) return true;
+    if (h->precision == SWOPT_PREC_BF16 && h->no_bf16_spectrum) return false;
     for (int i = 0; i < 2; ++i)
         if (h->tc_force_mt[i] || h->tc_force_ctas[i] || h->tc_force_ra[i] ||
             h->tc_force_split[i] || h->tc_force_nbuf[i])
@@ -314,16 +315,18 @@ bool route_fft(const swopt_handle* h)
 bool rounds(const swopt_handle* h) { return h->precision == SWOPT_PREC_BF16; }
 
 // What the selected precision's route needs (synchronises; never called while
-// capturing).
+// capturing).  Without memory for the spectrum of the BF16 kernel, also when the
+// tensor-core operator of another precision has made room, the tensor-core kernels
+// serve BF16, until a precision is selected again.
 swopt_status prepare_route(swopt_handle* h)
 {
     if (!use_tc(h)) return SWOPT_OK;
-    if (!route_fft(h)) return tc_prepare(h);
-    if (rounds(h) && !fft_prepare_bf16(h)) {
-        set_error("no memory for the spectrum of the BF16 kernel");
-        return SWOPT_ERR_OOM;
+    if (route_fft(h) && rounds(h) && !fft_prepare_bf16(h)) {
+        const bool room = h->tc != nullptr;
+        tc_release(h);
+        h->no_bf16_spectrum = !room || !fft_prepare_bf16(h);
     }
-    return SWOPT_OK;
+    return route_fft(h) ? SWOPT_OK : tc_prepare(h);
 }
 
 // The tensor-core operator of the selected precision, built if the spectral
@@ -1017,14 +1020,20 @@ swopt_status swopt_set_precision(swopt_handle* h, int precision)
     if (precision != SWOPT_PREC_FP32) {
         const int prev = h->precision;
         h->precision = precision;
+        h->no_bf16_spectrum = false;  // another try
         // a geometry that the tensor-core kernels refuse stays refused
         swopt_status s = tc_supported(h);
-        if (s == SWOPT_OK && route_fft(h)) tc_release(h);  // of another precision
         if (s == SWOPT_OK) s = prepare_route(h);
         if (s != SWOPT_OK) {
+            // back to the former precision, whose operator may have made room
+            char msg[sizeof(g_err)];
+            std::memcpy(msg, g_err, sizeof(msg));
             h->precision = prev;
+            prepare_route(h);
+            std::memcpy(g_err, msg, sizeof(msg));
             return s;
         }
+        if (route_fft(h)) tc_release(h);  // of another precision
     }
     h->precision = precision;
     return SWOPT_OK;

@@ -15,6 +15,7 @@ static int g_kernels;
 static size_t g_limit = (size_t)-1; /* an allocation above this many bytes fails */
 static long g_fail_in = -1;         /* the allocation after this many more fails */
 static long g_failed, g_live;
+static size_t g_largest;
 static cudaError_t g_last; /* until cudaGetLastError, as in the runtime */
 
 /* ---- control ---- */
@@ -26,6 +27,13 @@ void fake_reset(void)
     g_fail_in = -1;
     g_failed = 0;
     g_last = cudaSuccess;
+}
+/* the largest allocation asked for since the last call */
+size_t fake_largest(void)
+{
+    const size_t n = g_largest;
+    g_largest = 0;
+    return n;
 }
 void fake_limit(size_t bytes) { g_limit = bytes; }
 void fake_fail_in(long n) { g_fail_in = n; }
@@ -61,6 +69,7 @@ static cudaError_t launched(const void* fun, dim3 grid)
 cudaError_t cudaMalloc(void** p, size_t n)
 {
     *p = NULL;
+    if (n > g_largest) g_largest = n;
     if (n > g_limit || (g_fail_in >= 0 && g_fail_in-- == 0)) {
         ++g_failed;
         return g_last = cudaErrorMemoryAllocation;

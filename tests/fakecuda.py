@@ -27,6 +27,7 @@ def load(folder):
     for name, (args, res) in sw._SIGS.items():
         fn = getattr(L, name)
         fn.argtypes, fn.restype = args, res
+    L.fake_largest.restype = ctypes.c_size_t
     L.fake_limit.argtypes = [ctypes.c_size_t]
     L.fake_fail_in.argtypes = [ctypes.c_long]
     L.fake_failed.restype = L.fake_live.restype = L.fake_launches.restype = ctypes.c_long
@@ -61,6 +62,17 @@ class Handle:
     def prox_tv(self, iters=4):
         return self.L.swopt_prox_tv(self.h, self.c.ctypes.data, self.x.ctypes.data, 0.1, iters, 0,
                                     None)
+
+    def precision(self, name):
+        return self.L.swopt_set_precision(self.h, sw.PRECISION[name])
+
+    def pin(self):
+        """Ask for the tensor-core kernels, by a pinned schedule."""
+        for kernel in (0, 1):
+            assert self.L.swopt_tc_schedule(self.h, kernel, 1, 0) == 0
+
+    def adjoint(self):
+        return self.L.swopt_adjoint(self.h, self.y.ctypes.data, self.x.ctypes.data, None)
 
     def objective(self):
         F, fit = ctypes.c_double(), ctypes.c_double()

@@ -50,3 +50,59 @@ def test_tv_prox_after_a_failed_allocation(fake):
             assert fake.fake_launches(b"fgp_march") == before + 1
         finally:
             h.close()
+
+
+# a scan whose spectrum of the BF16 kernel takes more memory than the tensor-core
+# operator for BF16, and that one more than the operator for FP8
+SCAN = dict(X=40, Y=40, Z=60, T=200)
+
+
+def _largest(fake, precision, pinned):
+    """The largest array that a handle allocates to be used at the precision."""
+    h = fakecuda.Handle(fake, **SCAN)
+    if pinned:
+        h.pin()
+    fake.fake_largest()
+    assert h.precision(precision) == 0
+    h.close()
+    return fake.fake_largest()
+
+
+@pytest.mark.parametrize("first", ["fp32", "fp8"])
+def test_bf16_without_memory_for_its_spectrum(fake, first):
+    """The tensor-core kernels serve BF16 then, and the transforms again once
+    the precision is selected with enough memory."""
+    limit = _largest(fake, "bf16", False) - 1
+    assert limit >= _largest(fake, "bf16", True)
+    h = fakecuda.Handle(fake, **SCAN)
+    try:
+        assert h.precision(first) == 0
+        fake.fake_limit(limit)
+        assert h.precision("bf16") == 0, fake.swopt_last_error()
+        n = fake.fake_launches(b"spec_kernel"), fake.fake_launches(b"tc_conv_kernel")
+        assert h.forward() == 0 and h.adjoint() == 0
+        assert fake.fake_launches(b"spec_kernel") == n[0]
+        assert fake.fake_launches(b"tc_conv_kernel") == n[1] + 2
+        fake.fake_limit(2**63)
+        assert h.precision("bf16") == 0
+        assert h.forward() == 0 and h.adjoint() == 0
+        assert fake.fake_launches(b"spec_kernel") == n[0] + 2
+        assert fake.fake_launches(b"tc_conv_kernel") == n[1] + 2
+    finally:
+        h.close()
+
+
+def test_former_precision_serves_on_after_a_failed_selection(fake):
+    limit = _largest(fake, "fp8", True)
+    assert limit < _largest(fake, "bf16", True)
+    h = fakecuda.Handle(fake, **SCAN)
+    try:
+        h.pin()
+        assert h.precision("fp8") == 0
+        fake.fake_limit(limit)
+        assert h.precision("bf16") == OOM and b"cudaMalloc" in fake.swopt_last_error()
+        n = fake.fake_launches(b"tc_conv_kernel")
+        assert h.forward() == 0 and h.adjoint() == 0, fake.swopt_last_error()
+        assert fake.fake_launches(b"tc_conv_kernel") == n + 2
+    finally:
+        h.close()
