@@ -386,7 +386,7 @@ swopt_status normal_op(swopt_handle* h, const float* v, float* w, cudaStream_t s
     if (route_fft(h)) {
         FftImage img;
         img.out = w;
-        return fft_normal(h, v, nullptr, rounds(h), FftKeep::never, img, st);
+        return fft_normal(h, v, nullptr, rounds(h), false, img, st);
     }
     SW_TRY(apply_A(h, v, A_OUT_R, nullptr, nullptr, 1, st));
     SW_TRY(apply_AT(h, false, st));
@@ -406,8 +406,8 @@ swopt_status states_adjoint(swopt_handle* h, const float* y, cudaStream_t st)
     return apply_AT(h, true, st);
 }
 
-// h->g = A^T (C A P v - ytil), per state.  keep_u: h->u is written whatever the
-// measurements hold (see FftKeep).
+// h->g = A^T (C A P v - ytil), per state.  keep_u: ytil are not the bound
+// measurements' (see fft_normal).
 swopt_status state_gradient(swopt_handle* h, const float* v, const float* ytil, bool keep_u,
                             cudaStream_t st)
 {
@@ -415,8 +415,7 @@ swopt_status state_gradient(swopt_handle* h, const float* v, const float* ytil, 
         FftImage img;
         img.per_state = true;
         img.out = h->g;
-        return fft_normal(h, v, ytil, rounds(h), keep_u ? FftKeep::always : FftKeep::nonfinite, img,
-                          st);
+        return fft_normal(h, v, ytil, rounds(h), keep_u, img, st);
     }
     SW_TRY(apply_A(h, v, A_OUT_R, ytil, nullptr, 1, st));
     return apply_AT(h, false, st);
@@ -436,8 +435,7 @@ swopt_status refined_gradient(swopt_handle* h, const float* v, const float* ytil
         img.out = h->zin;
         img.xi = h->xi;
         img.G = h->G;
-        return fft_normal(h, v, ytil, rounds(h), ytil ? FftKeep::nonfinite : FftKeep::never, img,
-                          st);
+        return fft_normal(h, v, ytil, rounds(h), false, img, st);
     }
     SW_TRY(apply_A(h, v, A_OUT_R, ytil, nullptr, 1, st));
     SW_TRY(apply_AT(h, false, st));

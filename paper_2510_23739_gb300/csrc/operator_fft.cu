@@ -32,9 +32,16 @@
 //  * Scans wider than the largest transform are cut into overlapping tiles
 //    (L - 2 r outputs each).
 //
-// An output that is not finite is recomputed by the direct sum over its own
-// taps, so that an infinity or NaN in the input reaches the outputs whose
-// sums contain it and no others (a transform would spread it over the image).
+// A transform would spread an infinity, a NaN or a huge value (a mask of the
+// type's lowest one) of the input over the whole image.  The first pass of A and
+// of A^T therefore takes every value that is not below 2^64 out, as a zero, and
+// marks its scan position; the last pass adds such values' own terms to the
+// outputs within the support of a marked position.  So they reach the outputs
+// whose sums contain them and no others.  Without marks that costs a comparison per
+// value; one iteration of the largest workload (k = 31, 128^2 x 96, 0.89 ms) takes
+// 1.5 ms with NaNs or infinities at one pixel of the measurements and 2.6 ms with
+// nothing else in them.  Finite values from 2^64 cost the direct sums over what they
+// reach, and a solve spreads them: 1.2 s where one pixel holds 1e30.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -268,6 +275,7 @@ __device__ __forceinline__ void fft_line(const FftAxis& ax, float2* sm, Load loa
         fft_pass1<R, S>(ax.tw, ax.R2, n2, sm, lane, load)
     SW_RADIX(ax.R1, SW_P1)
 #undef SW_P1
+    if (S > 0) asm volatile("cp.async.wait_all;" ::: "memory");  // see fetch_marks
     __syncthreads();
 #define SW_P2(R)                                  \
     for (int k1 = warp; k1 < ax.R1; k1 += nw)     \
@@ -276,14 +284,21 @@ __device__ __forceinline__ void fft_line(const FftAxis& ax, float2* sm, Load loa
 #undef SW_P2
 }
 
-// True if any of the values is an infinity or NaN.
+// Values that the transforms do not take: infinities, NaNs and magnitudes from 2^64.
+// (What is below leaves 2^64 of FP32's range to the sums of the transforms.)
+constexpr float kHuge = 1.8446744e19f;
+
+__device__ __forceinline__ bool huge(float v) { return !(fabsf(v) < kHuge); }
+
+// True if any of the values is one.
 template <int R>
-__device__ __forceinline__ bool any_nonfinite(const float2 (&v)[R])
+__device__ __forceinline__ bool any_huge(const float2 (&v)[R])
 {
-    float s = 0.f;
+    float top = 0.f;  // the largest magnitude, or a NaN
 #pragma unroll
-    for (int i = 0; i < R; ++i) s = fmaf(v[i].x, 0.f, fmaf(v[i].y, 0.f, s));
-    return !(s == 0.f);
+    for (int i = 0; i < R; ++i)
+        asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(top) : "f"(v[i].x), "f"(v[i].y));
+    return huge(top);
 }
 
 // ---------------------------------------------------------------------------
@@ -301,7 +316,14 @@ struct FftShape {
     int round;      // operands rounded to BF16 (per state)
     int round2;
     const float* Sm;  // [Q][P][Z]
-    const float* Kf;  // [Z][k][k][Twp] FP32 kernel (direct sums of non-finite outputs)
+    const float* Kf;  // [Z][k][k][Twp] FP32 kernel (terms of the marked positions)
+    const int4* ftab; // banded groups of the kernel: depths per eight samples,
+    const int4* atab; // samples per eight depths (see Spec)
+    // Marked positions of A's and of A^T's input.  A mark is the tag of the call, one
+    // more than its predecessor's, so that nothing has to be cleared:
+    // marks[0] the call's tag, marks[1 + which] the last one with a marked position,
+    // then (from 4) [which][Y] the same per row and [which][Y][X] per position.
+    unsigned* marks;
     const int* gate;
     int want;
 };
@@ -339,50 +361,170 @@ __device__ __forceinline__ float folded(const FftShape& s, const float* __restri
     return acc;
 }
 
-// One output of A by its direct sum (the order and the zero blocks of
-// fwd_simt_kernel); only for outputs that the transforms made non-finite.
-__device__ __noinline__ float direct_forward(const FftShape& s, int round, const float* c, int m,
-                                             int y, int x, int w)
+enum { MARK_A = 0, MARK_AT = 1 };
+
+__device__ __forceinline__ unsigned* row_marks(const FftShape& s, int which)
 {
+    return s.marks + 4 + which * s.Y;
+}
+
+__device__ __forceinline__ unsigned* pos_marks(const FftShape& s, int which)
+{
+    return s.marks + 4 + 2 * s.Y + (size_t)which * s.Y * s.X;
+}
+
+// The call's tag: before its second launch has counted it (the first one marks
+// with it), and from then on.
+__device__ __forceinline__ unsigned next_tag(const FftShape& s) { return *(volatile unsigned*)s.marks + 1u; }
+__device__ __forceinline__ unsigned this_tag(const FftShape& s) { return *(volatile unsigned*)s.marks; }
+
+// The words marks[0 .. 2] into shared memory by the first thread: on their way during
+// the first pass, waited for before its barrier, and in no register until they are read.
+__device__ __forceinline__ void fetch_marks(const FftShape& s, uint4* words)
+{
+    if (threadIdx.x == 0)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(words)),
+                     "l"(s.marks)
+                     : "memory");
+}
+
+// True if the input of A or A^T has marked positions in this call.
+__device__ __forceinline__ bool any_mark(const uint4& words, int which)
+{
+    return words.x == (which == MARK_A ? words.y : words.z);
+}
+
+// The values of a thread's line entries, through shared-memory slots that only it
+// uses, around `f`: a call on values in registers would have the compiler spill them
+// on every path.
+template <int R, class F>
+__device__ __forceinline__ void through_slots(float2 (&v)[R], float2* slot, int stride, F f)
+{
+#pragma unroll
+    for (int i = 0; i < R; ++i) slot[i * stride] = v[i];
+    f();
+#pragma unroll
+    for (int i = 0; i < R; ++i) v[i] = slot[i * stride];
+}
+
+// Takes the huge values among line entries out, marking their positions (row y,
+// columns x0 + i step).
+__device__ __noinline__ void take_out(const FftShape& s, int which, unsigned tag, float2* slot, int stride,
+                                      int R, int y, int x0, int step)
+{
+    for (int i = 0; i < R; ++i) {
+        const float2 v = slot[i * stride];
+        if (!huge(v.x) && !huge(v.y)) continue;
+        pos_marks(s, which)[(size_t)y * s.X + x0 + i * step] = tag;
+        row_marks(s, which)[y] = tag;
+        s.marks[1 + which] = tag;
+        slot[i * stride] = make_float2(huge(v.x) ? 0.f : v.x, huge(v.y) ? 0.f : v.y);
+    }
+}
+
+// Calls f(dy, dx, position) for the marked positions that output (y, x) sums over
+// (SIGN 1: A, at (y + dy - r, x + dx - r); -1: A^T, at (y - dy + r, x - dx + r)).
+// f returns false to end.
+template <int SIGN, class F>
+__device__ __forceinline__ void marked_taps(const FftShape& s, int which, int y, int x, F f)
+{
+    const unsigned tag = this_tag(s);
+    const unsigned *rows = row_marks(s, which), *cells = pos_marks(s, which);
+    for (int dy = 0; dy < s.k; ++dy) {
+        const int yy = y + SIGN * (dy - s.r);
+        if (yy < 0 || yy >= s.Y || rows[yy] != tag) continue;
+        for (int dx = 0; dx < s.k; ++dx) {
+            const int xx = x + SIGN * (dx - s.r);
+            if (xx < 0 || xx >= s.X || cells[(size_t)yy * s.X + xx] != tag) continue;
+            if (!f(dy, dx, (size_t)yy * s.X + xx)) return;
+        }
+    }
+}
+
+// True if a row within the support of row y is marked.
+__device__ __forceinline__ bool marked_near(const FftShape& s, int which, int y)
+{
+    const unsigned tag = this_tag(s);
+    for (int yy = max(0, y - s.r); yy <= min(s.Y - 1, y + s.r); ++yy)
+        if (row_marks(s, which)[yy] == tag) return true;
+    return false;
+}
+
+// acc += value * kernel.  A value that is not finite also counts against a zero entry
+// of a block of eight that is not all zero, as in the direct kernels; block(i) is
+// entry i of that block.
+template <class Block>
+__device__ __forceinline__ void add_term(float& acc, float value, float kernel, int round, Block block)
+{
+    if (kernel == 0.f) {
+        if (isfinite(value)) return;
+        bool any = false;
+        for (int i = 0; i < 8; ++i) any |= block(i) != 0.f;
+        if (!any) return;
+    }
+    acc = fmaf(round_if(value, round), round_if(kernel, round), acc);
+}
+
+// The terms of the marked positions in one output of A (state m, sample w).  A sum
+// that is NaN stays so: it ends there, and the cost of NaNs with it.
+__device__ float marked_forward(const FftShape& s, int round, const float* c, int m, int y, int x, int w)
+{
+    const int4 band = s.ftab[w / kOG];
+    const size_t SZ = (size_t)s.Y * s.X * s.Z;
     float acc = 0.f;
-    for (int j = 0; j < s.Z; ++j)
-        for (int dy = 0; dy < s.k; ++dy)
-            for (int dx = 0; dx < s.k; ++dx) {
-                const int yy = y + dy - s.r, xx = x + dx - s.r;
-                if (yy < 0 || yy >= s.Y || xx < 0 || xx >= s.X) continue;
-                const float* kp = s.Kf + (((size_t)j * s.k + dy) * s.k + dx) * s.Twp;
+    marked_taps<1>(s, MARK_A, y, x, [&](int dy, int dx, size_t pos) {
+        for (int j = band.y; j < band.y + band.z; ++j) {
+            float b = 0.f;  // what the first pass took out
+            if (round) {
+                b = state_value(s, c, m, pos, j);
+                if (!huge(b)) continue;
+            } else {
                 bool any = false;
-                for (int i = 0; i < 8; ++i) any |= kp[(w & ~7) + i] != 0.f;
+                for (int p = 0; p < s.P; ++p) {
+                    const float v = c[p * SZ + pos * s.Z + j];
+                    if (!huge(v)) continue;
+                    any = true;
+                    b = fmaf(__ldg(s.Sm + ((size_t)m * s.P + p) * s.Z + j), v, b);
+                }
                 if (!any) continue;
-                const float b = state_value(s, c, m, (size_t)yy * s.X + xx, j);
-                acc = fmaf(round_if(b, round), round_if(kp[w], round), acc);
             }
+            const float* kp = s.Kf + (((size_t)j * s.k + dy) * s.k + dx) * s.Twp;
+            add_term(acc, b, kp[w], round, [&](int i) { return kp[(w & ~7) + i]; });
+            if (isnan(acc)) return false;
+        }
+        return true;
+    });
     return acc;
 }
 
-// One output of A^T (state m, depth j) by its direct sum over r, either the
-// residual [Q][Y][X][Twp] or (from_y) the measurements folded on the way.
-__device__ __noinline__ float direct_adjoint(const FftShape& s, int round, const float* r,
-                                             int from_y, int m, int y, int x, int j)
+// The same of A^T (depth j), for state m or, with m < 0, for species p (P^T over
+// the states); r is either the residual [Q][Y][X][Twp] or (from_y) the measurements.
+__device__ float marked_adjoint(const FftShape& s, int round, const float* r, int from_y, int m, int p,
+                                int y, int x, int j)
 {
+    const int4 band = s.atab[j / kOG];
     const int j8 = j & ~7;
+    const size_t kk = (size_t)s.k * s.k * s.Twp;
     float acc = 0.f;
-    for (int w = 0; w < s.Twp; ++w)
-        for (int dy = 0; dy < s.k; ++dy)
-            for (int dx = 0; dx < s.k; ++dx) {
-                const int yy = y - dy + s.r, xx = x - dx + s.r;
-                if (yy < 0 || yy >= s.Y || xx < 0 || xx >= s.X) continue;
-                const size_t tap = ((size_t)dy * s.k + dx) * s.Twp + w;
-                const size_t kk = (size_t)s.k * s.k * s.Twp;
-                bool any = false;
-                for (int i = 0; i < 8; ++i)
-                    any |= j8 + i < s.Z && s.Kf[(size_t)(j8 + i) * kk + tap] != 0.f;
-                if (!any) continue;
-                const size_t pos = (size_t)yy * s.X + xx;
-                const float v = from_y ? folded(s, r, m, pos, w)
-                                       : r[((size_t)m * s.Y * s.X + pos) * s.Twp + w];
-                acc = fmaf(round_if(v, round), round_if(s.Kf[(size_t)j * kk + tap], round), acc);
+    marked_taps<-1>(s, MARK_AT, y, x, [&](int dy, int dx, size_t pos) {
+        const float* kt = s.Kf + ((size_t)dy * s.k + dx) * s.Twp;
+        for (int q = m < 0 ? 0 : m; q < (m < 0 ? s.Q : m + 1); ++q) {
+            float sum = 0.f;
+            for (int w = band.y; w < band.y + band.z && !isnan(sum); ++w) {
+                const float v = from_y ? folded(s, r, q, pos, w)
+                                       : r[((size_t)q * s.Y * s.X + pos) * s.Twp + w];
+                if (!huge(v)) continue;
+                add_term(sum, v, kt[(size_t)j * kk + w], round, [&](int i) {
+                    return j8 + i < s.Z ? kt[(size_t)(j8 + i) * kk + w] : 0.f;
+                });
             }
+            if (sum == 0.f) continue;
+            acc = m < 0 ? fmaf(s.Sm[((size_t)q * s.P + p) * s.Z + j], sum, acc) : acc + sum;
+            if (isnan(acc)) return false;
+        }
+        return true;
+    });
     return acc;
 }
 
@@ -432,6 +574,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_forward_kernel(const 
     const size_t YX = (size_t)s.Y * s.X;
     const size_t row0 = (size_t)(row_ok ? gy : 0) * s.X;
     const bool two = ch + 1 < s.Z;
+    constexpr int kWhich = SRC == SRC_U || SRC == SRC_Y ? MARK_AT : MARK_A;
     // SRC_STATES: this thread's switching weights (its state and depths)
     float2 wt[kStates ? 8 : 1];
     if (kStates) {
@@ -497,6 +640,11 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_forward_kernel(const 
                     add(src + ((ptrdiff_t)(n * YX) + at) * s.T + t, (size_t)R2 * s.T, t + 1 < s.T,
                         none);
         }
+        if (any_huge(v)) {
+            float2* slot = sm + n2 * 32 + lane;
+            through_slots(v, slot, 32 * R2,
+                          [&] { take_out(s, kWhich, next_tag(s), slot, 32 * R2, R, gy, first, R2); });
+        }
         if (SRC != SRC_C && round) {
 #pragma unroll
             for (int i = 0; i < R; ++i) v[i] = make_float2(round_if(v[i].x, 1), round_if(v[i].y, 1));
@@ -518,6 +666,7 @@ struct YPass {
     unsigned width;     // Lx * C2
     unsigned items;     // plane-tiles * width
     unsigned items2;
+    int count;          // the second launch of a call: counts its tag
 };
 
 template <int S>
@@ -527,6 +676,8 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_y_kernel(const YPass a)
     const FftShape& s = a.s;
     grid_dependency();
     if (gated_off(s.gate, s.want)) return;
+    if (a.count && blockIdx.x == 0 && threadIdx.x == 0)
+        asm volatile("red.global.add.u32 [%0], 1;" ::"l"(s.marks) : "memory");
     const unsigned item = blockIdx.x * 32u + (threadIdx.x & 31);
     const bool ok = item < (second_variant(s) ? a.items2 : a.items);
     const unsigned col = item % a.width, pt = item / a.width;
@@ -557,14 +708,6 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_y_kernel(const YPass a)
 
 enum { IMG_STORE = 0, IMG_STEP = 1, IMG_REFINE = 2 };
 
-// Whether A's output u is in memory as A^T's direct sums would read it.
-enum { KEEP_NEVER = 0, KEEP_ALWAYS = 1, KEEP_NONFINITE = 2 };
-
-__device__ __forceinline__ bool kept(int keep, const double* ysq)
-{
-    return keep == KEEP_ALWAYS || (keep == KEEP_NONFINITE && !isfinite(*ysq));
-}
-
 struct XInverse {
     FftShape s;
     const float2* in;   // [plane][tile][rows_out][Lx][C2]
@@ -576,71 +719,62 @@ struct XInverse {
     // u: out = (scale ? Cm : 1) v - ytil
     const float* ytil;
     const float* Cmf;   // null: no scale
-    const float* c;     // input of A (direct sums)
+    const float* c;     // input of A (terms of its marked positions)
     // images: IMG_STORE out = v; IMG_STEP out = xi - alpha v; IMG_REFINE as pt_refine_kernel
     int add, add2;
     float alpha;
     const float* xi;
     float* G;
     const double* scal;
-    const float* r;     // input of A^T (direct sums): residual or measurements
-    int keep, keep2;    // whether r holds them (KEEP_*)
-    const double* ysq;
+    const float* r;     // input of A^T (the same): residual or measurements
     int from_y;
     int per_state;      // planes are states (else species, summed over the states)
 };
 
-// The values of a thread's second pass, through the shared-memory entries that
-// only it reads, around `fix`: a call on values in registers would have the
-// compiler spill them on every path.
-template <int R, class Fix>
-__device__ __forceinline__ void through_slots(float2 (&v)[R], float2* slot, Fix fix)
-{
-#pragma unroll
-    for (int i = 0; i < R; ++i) slot[i * 32] = v[i];
-    fix();
-#pragma unroll
-    for (int i = 0; i < R; ++i) v[i] = slot[i * 32];
-}
-
-// Entries i (column k1 + R1 i of the transform) of an image line that are not
-// finite, by their direct sums.
-__device__ __noinline__ void fix_image(const XInverse& a, float2* slot, int R, int k1, int R1,
-                                       int gx0, int gy, int plane, int ch)
+// The terms of marked positions in the image line that a thread has written, added
+// to what it wrote (the line of row gy, tile columns from gx0, channels ch and
+// ch + 1).  At the end of the kernel, where no value of the transform is live.
+template <int MODE>
+__device__ __noinline__ void add_marked_image(const XInverse& a, int gx0, int gy, int plane, int ch)
 {
     const FftShape& s = a.s;
+    if (!marked_near(s, MARK_AT, gy)) return;
     const int round = second_variant(s) ? s.round2 : s.round;
-    for (int i = 0; i < R; ++i) {
-        const int o = k1 + R1 * i - s.x.pad, gx = gx0 + o;
-        if (o < 0 || o >= s.x.out || gx >= s.X) continue;
-        for (int h = 0; h < 2 && ch + h < s.Z; ++h) {
-            float* p = reinterpret_cast<float*>(slot + i * 32) + h;
-            if (isfinite(*p)) continue;
-            float acc = 0.f;
-            if (a.per_state) {
-                acc = direct_adjoint(s, round, a.r, a.from_y, plane, gy, gx, ch + h);
-            } else {
-                for (int m = 0; m < s.Q; ++m)
-                    acc = fmaf(s.Sm[((size_t)m * s.P + plane) * s.Z + ch + h],
-                               direct_adjoint(s, round, a.r, a.from_y, m, gy, gx, ch + h), acc);
+    const float beta = MODE == IMG_REFINE ? (float)a.scal[1] : 0.f;
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int k1 = warp; k1 < s.x.R1; k1 += nw)
+        for (int i = 0; i < s.x.R2; ++i) {
+            const int o = k1 + s.x.R1 * i - s.x.pad, gx = gx0 + o;
+            if (o < 0 || o >= s.x.out || gx >= s.X) continue;
+            for (int h = 0; h < 2 && ch + h < s.Z; ++h) {
+                const float t = marked_adjoint(s, round, a.r, a.from_y, a.per_state ? plane : -1, plane,
+                                               gy, gx, ch + h);
+                const size_t at = (((size_t)plane * s.Y + gy) * s.X + gx) * s.Z + ch + h;
+                if (MODE == IMG_REFINE) a.G[at] += t;
+                a.out[at] = MODE == IMG_STORE ? a.out[at] + t : fmaf(-a.alpha, fmaf(beta, t, t), a.out[at]);
             }
-            *p = acc;
         }
-    }
 }
 
-// The same for a line of u: columns x0 + k1 + R1 i.
-__device__ __noinline__ void fix_u(const FftShape& s, int round, const float* c, float2* slot, int R,
-                                   int k1, int R1, int x0, int end, int gy, int m, int w)
+// The same for a line of u (state m, samples w and w + 1): u += factor * terms, or with
+// `from` u = from + factor * terms (null: of zero).
+__device__ __noinline__ void add_marked_u(const FftShape& s, int round, const float* c, float factor,
+                                          const float* from, bool in_place, float* u, int gx0, int gy,
+                                          int m, int w)
 {
-    for (int i = 0; i < R; ++i) {
-        const int gx = x0 + k1 + R1 * i;
-        if (gx < max(0, x0 + s.x.pad) || gx >= end) continue;
-        for (int h = 0; h < 2; ++h) {
-            float* p = reinterpret_cast<float*>(slot + i * 32) + h;
-            if (!isfinite(*p)) *p = direct_forward(s, round, c, m, gy, gx, w + h);
+    const bool near = marked_near(s, MARK_A, gy);
+    if (in_place && !near) return;
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int k1 = warp; k1 < s.x.R1; k1 += nw)
+        for (int i = 0; i < s.x.R2; ++i) {
+            const int o = k1 + s.x.R1 * i - s.x.pad, gx = gx0 + o;
+            if (o < 0 || o >= s.x.out || gx >= s.X) continue;
+            const size_t at = (((size_t)m * s.Y + gy) * s.X + gx) * s.Twp + w;
+            for (int h = 0; h < 2; ++h) {
+                const float t = near ? marked_forward(s, round, c, m, gy, gx, w + h) : 0.f;
+                u[at + h] = fmaf(factor, t, in_place ? u[at + h] : from ? from[at + h] : 0.f);
+            }
         }
-    }
 }
 
 // A^T's inverse along x: images [plane][Y][X][Z].
@@ -664,7 +798,9 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
     const float2* in = a.in + (size_t)line * s.x.L * a.C2 + q;
     const float beta = MODE == IMG_REFINE ? (float)a.scal[1] : 0.f;
     const bool alt = second_variant(s);
-    const int add = alt ? a.add2 : a.add, keep = alt ? a.keep2 : a.keep;
+    const int add = alt ? a.add2 : a.add;
+    __shared__ uint4 words;
+    fetch_marks(s, &words);
     const bool two = ch + 1 < s.Z;
     fft_line<1>(
         s.x, sm,
@@ -681,10 +817,6 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
                 const int o = k1 + R1 * i - s.x.pad, gx = gx0 + o;
                 return o >= 0 && o < s.x.out && gx < s.X ? gx : -1;
             };
-            if (any_nonfinite(v) && kept(keep, a.ysq)) {
-                float2* slot = sm + k1 * R * 32 + (threadIdx.x & 31);
-                through_slots(v, slot, [&] { fix_image(a, slot, R, k1, R1, gx0, gy, plane, ch); });
-            }
             const size_t base = ((size_t)plane * YX + (size_t)gy * s.X) * s.Z + ch;
             auto at = [&](int gx) { return base + (size_t)gx * s.Z; };
             auto get = [&](const float* p) {
@@ -729,6 +861,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
                 }
             }
         });
+    if (row_ok && any_mark(words, MARK_AT)) add_marked_image<MODE>(a, gx0, gy, plane, ch);
 }
 
 // A's inverse along x: u [Q][Y][X][Twp], the scaled folded residual, zero past
@@ -750,6 +883,8 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_u_kernel(const XInver
     const int w = 2 * (int)q;
     const float2* in = a.in + (size_t)line * s.x.L * a.C2 + q;
     const float cm = ok && a.Cmf ? a.Cmf[m] : 1.f;
+    __shared__ uint4 words;
+    fetch_marks(s, &words);
     fft_line<1>(
         s.x, sm,
         [&](auto& v, int n2, int R2) {
@@ -774,28 +909,23 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_u_kernel(const XInver
                                                 a.ytil + base + (size_t)gx * s.Twp))
                                           : make_float2(0.f, 0.f);
             }
-            if (any_nonfinite(v)) {
-                float2* slot = sm + k1 * R * 32 + (threadIdx.x & 31);
-                through_slots(v, slot, [&] {
-                    fix_u(s, s.round, a.c, slot, R, k1, R1, gx0 - s.x.pad, min(s.X, gx0 + s.x.out), gy,
-                          m, w);
-                });
-            }
 #pragma unroll
             for (int i = 0; i < R; ++i)
                 if (const int gx = out_x(i); gx >= 0)
                     *reinterpret_cast<float2*>(a.out + base + (size_t)gx * s.Twp) =
                         make_float2(fmaf(cm, v[i].x, -yt[i].x), fmaf(cm, v[i].y, -yt[i].y));
         });
+    if (row_ok && in_ok && any_mark(words, MARK_A))
+        add_marked_u(s, s.round, a.c, cm, nullptr, true, a.out, gx0, gy, m, w);
 }
 
 // A's inverse along x, the scaled folded residual, and A^T's forward along x in
 // one pass (one tile): u stays in registers.  The inverse's second DFTs leave
 // x = k1 + R1 k2 in the thread that needs exactly these for a first DFT of the
-// transform taken as L = R2 R1, so the two transforms share that step.  u is
-// written too when `keep` asks for it (the direct sums of A^T read it if the
-// measurements hold infinities or NaNs).  Against the two kernels it replaces
-// it saves a write and a read of u.
+// transform taken as L = R2 R1, so the two transforms share that step.  Against the
+// two kernels it replaces it saves a write and a read of u.  u is written too, and
+// its huge values taken out, where they can come from the input: A's has marked
+// positions, or the measurements hold values from 2^48 (by the sum of their squares).
 struct XResidual {
     FftShape s;
     const float2* in;   // [state][Y][Lx][C2]
@@ -806,12 +936,13 @@ struct XResidual {
     const float* Cmf;
     const float* c;
     float* u;
-    int keep;           // KEEP_*
-    const double* ysq;  // KEEP_NONFINITE: sum of squares of the measurements
+    int keep;           // u is written in any case
+    const double* ysq;  // sum of squares of the measurements behind ytil
     const float* ytil2;
     const float* c2;
-    int keep2;
 };
+
+constexpr double kHugeYsq = 7.9228162514264338e28;  // 2^96
 
 // 112 registers: three blocks of 6 warps per SM, without spills
 __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual a)
@@ -833,7 +964,10 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
     const bool alt = second_variant(s);
     const float* ytil = alt ? a.ytil2 : a.ytil;
     const int round = alt ? s.round2 : s.round;
-    const bool keep = kept(alt ? a.keep2 : a.keep, a.ysq);
+    __shared__ uint4 words;
+    __shared__ int s_keep;
+    fetch_marks(s, &words);
+    if (threadIdx.x == 0) s_keep = a.keep || (ytil && !(*a.ysq < kHugeYsq));
     const size_t base = (((size_t)m * s.Y + row) * s.X) * s.Twp + w;
     auto load = [&](auto& v, int n2, int R2) {
         constexpr int R = sizeof(v) / sizeof(v[0]);
@@ -846,9 +980,17 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
         fft_pass1<R, 1>(ax.tw, ax.R2, n2, sm, lane, load)
     SW_RADIX(ax.R1, SW_P1)
 #undef SW_P1
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    const bool marked = any_mark(words, MARK_A);
+    // the marked positions' terms join ytil, in the place of u
+    if (ok && marked) {
+        add_marked_u(s, round, alt ? a.c2 : a.c, -cm, ytil, false, a.u, 0, row, m, w);
+        ytil = a.u;
+    }
     auto middle = [&](auto& v, int k1, int R1) {
         constexpr int R = sizeof(v) / sizeof(v[0]);
+        const bool keep = marked || s_keep;
         float2 yt[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) {
@@ -857,18 +999,22 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
                                                    ytil + base + (size_t)gx * s.Twp))
                                              : make_float2(0.f, 0.f);
         }
-        if (ok && any_nonfinite(v)) {
-            float2* slot = sm + k1 * R * 32 + lane;
-            through_slots(v, slot, [&] { fix_u(s, round, alt ? a.c2 : a.c, slot, R, k1, R1, 0, s.X, row, m, w); });
-        }
 #pragma unroll
         for (int i = 0; i < R; ++i) {
             const int gx = k1 + R1 * i;
             v[i] = make_float2(fmaf(cm, v[i].x, -yt[i].x), fmaf(cm, v[i].y, -yt[i].y));
             if (keep && ok && gx < s.X)
                 *reinterpret_cast<float2*>(a.u + base + (size_t)gx * s.Twp) = v[i];
-            if (round) v[i] = make_float2(round_if(v[i].x, 1), round_if(v[i].y, 1));
             if (gx >= s.X) v[i] = make_float2(0.f, 0.f);
+        }
+        if (keep && ok && any_huge(v)) {
+            float2* slot = sm + k1 * R * 32 + lane;
+            through_slots(v, slot, 32,
+                          [&] { take_out(s, MARK_AT, this_tag(s), slot, 32, R, row, k1, R1); });
+        }
+        if (round) {
+#pragma unroll
+            for (int i = 0; i < R; ++i) v[i] = make_float2(round_if(v[i].x, 1), round_if(v[i].y, 1));
         }
         Dft<R, -1>::run(v);
         // into the entries that this thread has read
@@ -1369,6 +1515,7 @@ struct FftOperator {
     float2* KA[2] = {nullptr, nullptr};
     BandEntry* band = nullptr;
     int nband = 0;
+    unsigned* marks = nullptr;  // see FftShape
     float2* w0 = nullptr;    // workspaces, the spectra before and after a pass
     float2* w1 = nullptr;
     int fchunk = 2, achunk = 2;  // states per block of the two products
@@ -1440,6 +1587,7 @@ void fft_release(swopt_handle* h)
         cudaFree(f->KA[i]);
     }
     cudaFree(f->band);
+    cudaFree(f->marks);
     cudaFree(f->w0);
     cudaFree(f->w1);
     delete f;
@@ -1599,10 +1747,13 @@ void fft_prepare(swopt_handle* h)
     };
     // A's input side and A^T's per-state output side hold depths, the other samples
     const size_t area = (size_t)by.L * bx.L;
+    const size_t marks = 4 + 2 * (size_t)h->Y * (1 + h->X);
     const size_t ws = (size_t)f->tiles * area * std::max(h->Q, h->P) * std::max(Cz2, Ct2);
     const bool ok = upload(&f->ftab, ft) && upload(&f->atab, at) && upload(&f->band, band) &&
                     upload(&f->twy, roots(by.L)) && upload(&f->twx, roots(bx.L)) &&
                     try_alloc(&f->w0, ws) && try_alloc(&f->w1, ws) &&
+                    try_alloc(&f->marks, marks) &&
+                    cudaMemset(f->marks, 0, marks * sizeof(unsigned)) == cudaSuccess &&
                     try_alloc(&f->S4, (size_t)h->Z * h->Q * ((h->P + 3) / 4)) &&
                     fft_weights(h) == SWOPT_OK && build_spectrum(h, 0);
     f->y.tw = f->twy;
@@ -1632,6 +1783,7 @@ FftShape shape_of(const swopt_handle* h, bool round)
     s.sel = nullptr;
     s.round = s.round2 = round ? 1 : 0;
     s.Sm = h->Sm; s.Kf = h->Kf;
+    s.ftab = f->ftab; s.atab = f->atab; s.marks = f->marks;
     s.gate = h->gate; s.want = h->gate_want;
     return s;
 }
@@ -1654,7 +1806,7 @@ swopt_status launch_lines(swopt_handle* h, void (*kernel)(const Args), const Arg
 }
 
 swopt_status launch_y(swopt_handle* h, const FftShape& s, bool inverse, int planes, int planes2, int C2,
-                      const float2* in, float2* out, cudaStream_t st)
+                      const float2* in, float2* out, bool count, cudaStream_t st)
 {
     YPass a{};
     a.s = s;
@@ -1663,6 +1815,7 @@ swopt_status launch_y(swopt_handle* h, const FftShape& s, bool inverse, int plan
     a.width = (unsigned)(s.x.L * C2);
     a.items = (unsigned)(planes * s.tiles) * a.width;
     a.items2 = (unsigned)(planes2 * s.tiles) * a.width;
+    a.count = count ? 1 : 0;
     return launch_lines(h, inverse ? fft_y_kernel<1> : fft_y_kernel<-1>, a,
                         std::max(a.items, a.items2), s.y, st);
 }
@@ -1743,23 +1896,24 @@ swopt_status forward_to_lines(swopt_handle* h, const FftShape& s, const float* c
                         : s.round ? fft_x_forward_kernel<SRC_STATES>
                                   : fft_x_forward_kernel<SRC_C>,
                         a, std::max(a.items, a.items2), f->x, st));
-    SW_TRY(launch_y(h, s, false, planes, planes2, f->Cz2, f->w0, f->w1, st));
+    SW_TRY(launch_y(h, s, false, planes, planes2, f->Cz2, f->w0, f->w1, true, st));
     if (gated) SW_TRY((launch_spec<false, MAP_GATED>(h, s, f->w1, f->w0, st)));
     else if (s.round) SW_TRY((launch_spec<false, MAP_NONE>(h, s, f->w1, f->w0, st)));
     else SW_TRY((launch_spec<false, MAP_SPECIES>(h, s, f->w1, f->w0, st)));
-    return launch_y(h, s, true, h->Q, h->Q, f->Ct2, f->w0, f->w1, st);
+    return launch_y(h, s, true, h->Q, h->Q, f->Ct2, f->w0, f->w1, false, st);
 }
 
 // The lines of A^T's input, transformed along x in f->w0 -> the image outputs.
+// first: the launch before this was the call's first one.
 swopt_status adjoint_from_lines(swopt_handle* h, const FftShape& s, const float* r, bool from_y,
-                                int keep, int keep2, const FftImage& img, cudaStream_t st)
+                                bool first, const FftImage& img, cudaStream_t st)
 {
     FftOperator* f = h->fft;
-    SW_TRY(launch_y(h, s, false, h->Q, h->Q, f->Ct2, f->w0, f->w1, st));
+    SW_TRY(launch_y(h, s, false, h->Q, h->Q, f->Ct2, f->w0, f->w1, first, st));
     if (img.per_state) SW_TRY((launch_spec<true, MAP_NONE>(h, s, f->w1, f->w0, st)));
     else SW_TRY((launch_spec<true, MAP_SPECIES>(h, s, f->w1, f->w0, st)));
     const int planes = img.per_state ? h->Q : h->P;
-    SW_TRY(launch_y(h, s, true, planes, planes, f->Cz2, f->w0, f->w1, st));
+    SW_TRY(launch_y(h, s, true, planes, planes, f->Cz2, f->w0, f->w1, false, st));
     XInverse v{};
     v.s = s;
     v.in = f->w1;
@@ -1773,9 +1927,6 @@ swopt_status adjoint_from_lines(swopt_handle* h, const FftShape& s, const float*
     v.G = img.G;
     v.scal = h->scal;
     v.r = r;
-    v.keep = keep;
-    v.keep2 = keep2;
-    v.ysq = h->scal + kScalYsq;
     v.from_y = from_y ? 1 : 0;
     v.per_state = img.per_state ? 1 : 0;
     v.vec = (h->Z % 2) == 0 && aligned8(img.out) && aligned8(img.xi) && aligned8(img.G);
@@ -1827,17 +1978,12 @@ swopt_status fft_adjoint(swopt_handle* h, const float* src, bool from_y, bool ro
     prof_begin(h, 1, st, &rec);
     SW_TRY(launch_lines(h, from_y ? fft_x_forward_kernel<SRC_Y> : fft_x_forward_kernel<SRC_U>, a,
                         a.items, f->x, st));
-    SW_TRY(adjoint_from_lines(h, s, src, from_y, KEEP_ALWAYS, KEEP_ALWAYS, img, st));
+    SW_TRY(adjoint_from_lines(h, s, src, from_y, true, img, st));
     prof_end(h, &rec, st);
     return SWOPT_OK;
 }
 
 namespace {
-
-int keep_of(FftKeep k)
-{
-    return k == FftKeep::always ? KEEP_ALWAYS : k == FftKeep::never ? KEEP_NEVER : KEEP_NONFINITE;
-}
 
 // From the lines of A in f->w1 through the residual to A^T's output.
 swopt_status residual_to_image(swopt_handle* h, const FftShape& s, const XResidual& args,
@@ -1861,12 +2007,12 @@ swopt_status residual_to_image(swopt_handle* h, const FftShape& s, const XResidu
     const int warps = std::max(f->x.R1, f->x.R2) == 9 ? 9 : fft_warps(f->x);
     SW_CUDA(launch_pdl(fft_x_residual_kernel, (v.items + 31) / 32, 32 * warps, smem, st, v));
     SW_LAUNCHED(h);
-    return adjoint_from_lines(h, s, h->u, false, v.keep, v.keep2, img, st);
+    return adjoint_from_lines(h, s, h->u, false, false, img, st);
 }
 
 }  // namespace
 
-swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool round, FftKeep keep,
+swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool round, bool keep_u,
                         const FftImage& img, cudaStream_t st)
 {
     if (h->fft->tiles > 1) {
@@ -1882,7 +2028,7 @@ swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool
     XResidual v{};
     v.ytil = v.ytil2 = ytil;
     v.c = v.c2 = c;
-    v.keep = v.keep2 = keep_of(keep);
+    v.keep = keep_u ? 1 : 0;
     SW_TRY(residual_to_image(h, s, v, img, st));
     prof_end(h, &rec, st);
     return SWOPT_OK;
@@ -1929,8 +2075,6 @@ swopt_status fft_refine(swopt_handle* h, const float* delta, const float* c, con
     v.ytil2 = ytil;
     v.c = delta;
     v.c2 = c;
-    v.keep = KEEP_NEVER;
-    v.keep2 = KEEP_NONFINITE;
     SW_TRY(residual_to_image(h, s, v, img, st));
     end();
     return SWOPT_OK;

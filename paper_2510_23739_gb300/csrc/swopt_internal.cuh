@@ -382,12 +382,10 @@ struct FftImage {
 // [N][Y][X][T] folded on the way.
 swopt_status fft_adjoint(swopt_handle* h, const float* src, bool from_y, bool round,
                          const FftImage& img, cudaStream_t st);
-// A^T (C A P c - ytil) without u in between.  keep: whether h->u is written
-// too, as the direct sums need it where the result is not finite: always, or
-// only if the bound measurements (scal[kScalYsq]) hold infinities or NaNs; never
-// leaves such results NaN.
-enum class FftKeep { never, always, nonfinite };
-swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool round, FftKeep keep,
+// A^T (C A P c - ytil) without u in between.  ytil: the bound measurements' (of
+// which scal[kScalYsq] tells whether they hold huge values), null, or with keep_u any
+// others (h->u is written then in any case).
+swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool round, bool keep_u,
                         const FftImage& img, cudaStream_t st);
 // The refined solve's step decided on the device, in one chain of launches: by
 // h->sched[0], 0: G += H^T H delta with operands rounded if `round`; else
