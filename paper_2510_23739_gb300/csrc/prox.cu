@@ -749,53 +749,120 @@ __global__ void fista_scalars_kernel(double* scal, int mode)
 __global__ void set_scalar_kernel(double* scal, int slot, double v) { scal[slot] = v; }
 
 // ---- deterministic FP64 reductions (pass 1: fixed grid; pass 2: one block) ----
-// Sums of products over long arrays.  FP64 arithmetic and conversions run at
-// 1/64 of the FP32 rate here: with one of each per element the sum of squares
-// of 0.42 GB took 474 us.  So a thread sums 16 products exactly enough in FP32
-// pairs first (product and its error by FMA, sum and its error by Knuth's
-// two-sum; what is dropped is below 2^-43 of the 16) and adds the pair to its
-// FP64 sum: 83 us.  Products that would leave FP32's range take FP64 throughout.
-struct PairSum {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float x, float y)
+// Sums of products over long arrays, to FP64's accuracy.  FP64 arithmetic and
+// conversions run at 1/64 of the FP32 rate here: with one of each per element the
+// sum of squares of 0.42 GB took 474 us.  So a thread carries its sum as three FP32
+// terms over up to 128 products (a product and its error by FMA, sums and their errors
+// by Knuth's two-sum; only errors of the third term are dropped, 2^-58 of the products)
+// and adds them to FP64 then: the two sums of an objective over 0.42 GB of y and 0.17 GB
+// of u take 107 us (87 us with two terms, whose sums of 64 squares were off by up to
+// 4e-14).  Even and odd products have a sum each, as the halves of packed FP32
+// instructions.  Against the exact sum of 64 squares of normal
+// numbers: 1.0e-16, where 64 FP64 additions have 7.7e-16 (the worst of 60).
+// Groups whose largest product leaves [2^-80, 2^120], where an error or a sum would
+// leave FP32's range, and those with infinities and NaNs take FP64 throughout.
+constexpr float kProductLow = 8.2718061e-25f;   // 2^-80
+constexpr float kProductHigh = 1.3292280e36f;   // 2^120
+constexpr int kSumGroups = 8;                   // groups of 16 between two FP64 additions
+
+__device__ __forceinline__ float two_sum(float a, float b, float& err)
+{
+    const float t = a + b, z = t - a;
+    err = (a - (t - z)) + (b - z);
+    return t;
+}
+
+// Two FP32 numbers in one register pair.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack(-1.f, -1.f), a); }
+__device__ __forceinline__ f32x2 two_sum2(f32x2 a, f32x2 b, f32x2& err)
+{
+    const f32x2 t = add2(a, b), z = sub2(t, a);
+    err = add2(sub2(a, sub2(t, z)), sub2(b, z));
+    return t;
+}
+
+struct ProductSum {
+    f32x2 s = 0, c = 0, d = 0;
+    int groups = 0;
+    double total = 0.0;
+
+    __device__ __forceinline__ void flush()
     {
-        const float p = x * y, e = fmaf(x, y, -p);
-        const float t = s + p, z = t - s;
-        c += ((s - (t - z)) + (p - z)) + e;
-        s = t;
+        const float2 s2 = unpack(s), c2 = unpack(c), d2 = unpack(d);
+        float e1, e2, e3;
+        const float hi = two_sum(s2.x, s2.y, e1);
+        const float mid = two_sum(two_sum(c2.x, c2.y, e2), e1, e3);
+        total += (double)hi + ((double)mid + (double)((d2.x + d2.y) + (e2 + e3)));
+        s = c = d = 0;
+        groups = 0;
+    }
+    __device__ __forceinline__ void add(const float (&x)[16], const float (&y)[16])
+    {
+        float top = 0.f;  // the largest magnitude, or a NaN
+        f32x2 p[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            p[i] = mul2(pack(x[2 * i], x[2 * i + 1]), pack(y[2 * i], y[2 * i + 1]));
+            const float2 v = unpack(p[i]);
+            asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(top) : "f"(v.x), "f"(v.y));
+        }
+        if (top >= kProductLow && top <= kProductHigh) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const f32x2 e = fma2(pack(x[2 * i], x[2 * i + 1]), pack(y[2 * i], y[2 * i + 1]),
+                                     mul2(p[i], pack(-1.f, -1.f)));
+                f32x2 e1, e2, e3;
+                s = two_sum2(s, p[i], e1);
+                const f32x2 g = two_sum2(e1, e, e2);
+                c = two_sum2(c, g, e3);
+                d = add2(d, add2(e2, e3));
+            }
+            if (++groups == kSumGroups) flush();
+            return;
+        }
+        bool zero = true;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) zero = zero && (x[i] == 0.f || y[i] == 0.f);
+        if (zero && top == 0.f) return;
+        for (int i = 0; i < 16; ++i) total += (double)x[i] * (double)y[i];
+    }
+    __device__ __forceinline__ double value()
+    {
+        flush();
+        return total;
     }
 };
-
-constexpr float kPairLow = 9.094947e-13f;  // 2^-40
-constexpr float kPairHigh = 1.15292150e18f;  // 2^60
-
-// True if the pair arithmetic holds for products of values up to amax.
-__device__ __forceinline__ bool pair_range(float amax)
-{
-    return amax == 0.f || (amax >= kPairLow && amax <= kPairHigh);
-}
-
-template <int N>
-__device__ __forceinline__ double sum_products(const float (&x)[N], const float (&y)[N])
-{
-    float ax = 0.f, ay = 0.f;
-    bool fine = true;  // fmaxf drops NaNs
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        ax = fmaxf(ax, fabsf(x[i]));
-        ay = fmaxf(ay, fabsf(y[i]));
-        fine = fine && x[i] == x[i] && y[i] == y[i];
-    }
-    if (fine && pair_range(ax) && pair_range(ay)) {
-        PairSum p;
-#pragma unroll
-        for (int i = 0; i < N; ++i) p.add(x[i], y[i]);
-        return (double)p.s + (double)p.c;
-    }
-    double s = 0.0;
-    for (int i = 0; i < N; ++i) s += (double)x[i] * (double)y[i];
-    return s;
-}
 
 // sum x y (x == y: sum of squares, read once); 16-byte loads over the first
 // n16 * 16 entries (0 if an array is not 16-byte aligned)
@@ -804,7 +871,7 @@ __global__ void __launch_bounds__(kRedThreads) red_dot_kernel(const float* __res
                                                               size_t n, size_t n16, double* parts)
 {
     __shared__ double sh[kRedThreads / 32];
-    double s = 0.0;
+    ProductSum sum;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     // group g of 16: float4s g % 32 + 128 (g / 32) + {0, 32, 64, 96}, so that the
@@ -820,16 +887,17 @@ __global__ void __launch_bounds__(kRedThreads) red_dot_kernel(const float* __res
             a[4 * i] = v.x; a[4 * i + 1] = v.y; a[4 * i + 2] = v.z; a[4 * i + 3] = v.w;
         }
         if (x == y) {
-            s += sum_products(a, a);
+            sum.add(a, a);
         } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float4 v = __ldg(y4 + 32 * i);
                 b[4 * i] = v.x; b[4 * i + 1] = v.y; b[4 * i + 2] = v.z; b[4 * i + 3] = v.w;
             }
-            s += sum_products(a, b);
+            sum.add(a, b);
         }
     }
+    double s = sum.value();
     for (size_t i = 16 * n16 + first; i < n; i += stride) s += (double)x[i] * (double)y[i];
     s = block_sum(s, sh);
     if (threadIdx.x == 0) parts[blockIdx.x] = s;
@@ -844,7 +912,7 @@ __global__ void __launch_bounds__(kRedThreads) red_states_kernel(const float* __
 {
     __shared__ double sh[kRedThreads / 32];
     const float* xm = x + (size_t)blockIdx.y * n;
-    double s = 0.0;
+    ProductSum sum;
     for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < n / 16;
          g += (size_t)gridDim.x * blockDim.x) {
         float a[16];
@@ -853,9 +921,9 @@ __global__ void __launch_bounds__(kRedThreads) red_states_kernel(const float* __
             const float4 v = __ldg(reinterpret_cast<const float4*>(xm) + 4 * g + i);
             a[4 * i] = v.x; a[4 * i + 1] = v.y; a[4 * i + 2] = v.z; a[4 * i + 3] = v.w;
         }
-        s += sum_products(a, a);
+        sum.add(a, a);
     }
-    s = block_sum(s, sh);
+    const double s = block_sum(sum.value(), sh);
     if (threadIdx.x == 0) parts[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = s * (double)w[blockIdx.y];
 }
 
@@ -1040,7 +1108,7 @@ __global__ void __launch_bounds__(128) param_partial_kernel(const float* __restr
         const float* gm = g + (size_t)m * S * Z + j;
         for (int p = p0; p < min(P, p0 + 4); ++p) {
             const float* cp = c + (size_t)p * S * Z + j;
-            double w = 0.0;
+            ProductSum sum;
             int q = s0;
             for (; q + 16 <= s1; q += 16) {
                 float x[16], y[16];
@@ -1049,8 +1117,9 @@ __global__ void __launch_bounds__(128) param_partial_kernel(const float* __restr
                     x[i] = __ldg(gm + (size_t)(q + i) * Z);
                     y[i] = __ldg(cp + (size_t)(q + i) * Z);
                 }
-                w += sum_products(x, y);
+                sum.add(x, y);
             }
+            double w = sum.value();
             for (; q < s1; ++q) w += (double)gm[(size_t)q * Z] * (double)cp[(size_t)q * Z];
             parts[(((size_t)blockIdx.x * Q + m) * P + p) * Z + j] = w;
         }
