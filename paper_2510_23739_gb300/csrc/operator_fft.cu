@@ -1686,6 +1686,9 @@ void fft_prepare(swopt_handle* h)
     // this estimate: few are preferred (one H^T H at 128^2 x 96 in 4 x 4 tiles 717 us,
     // in one 417; 64^2 x 64 139 and 92)
     const double states = 8.0;
+    // channel pairs of all planes, on the side where they are most: samples of the
+    // states, or depths of the states or species
+    const size_t planes = std::max((size_t)h->Q * Ct2, (size_t)std::max(h->Q, h->P) * Cz2);
     double best = 1e300;
     FftAxis by{}, bx{};
     for (const Length& ly : kLengths)
@@ -1696,7 +1699,7 @@ void fft_prepare(swopt_handle* h)
             const double kbytes = 0.5 * area * (frows + arows) * kOG * 8.0;
             const double sbytes = tiles * area * 8.0 * 8.0 * (h->P * Cz2 + states * Ct2);
             const double flops = tiles * 0.5 * area * (frows + arows) * kOG * 8.0 * states;
-            const double work = 8.0 * tiles * area * std::max(h->Q * Ct2, h->Q * Cz2);
+            const double work = 8.0 * tiles * area * (double)planes;
             // memory limits: 24 GB of K^ (twice with the BF16 one), 8 GB per workspace
             if (kbytes > 24e9 || work > 8e9) continue;
             double t = std::max(kbytes / 5e12, flops / 40e12) + sbytes / 5e12;
@@ -1745,10 +1748,9 @@ void fft_prepare(swopt_handle* h)
         }
         return w;
     };
-    // A's input side and A^T's per-state output side hold depths, the other samples
     const size_t area = (size_t)by.L * bx.L;
     const size_t marks = 4 + 2 * (size_t)h->Y * (1 + h->X);
-    const size_t ws = (size_t)f->tiles * area * std::max(h->Q, h->P) * std::max(Cz2, Ct2);
+    const size_t ws = (size_t)f->tiles * area * planes;
     const bool ok = upload(&f->ftab, ft) && upload(&f->atab, at) && upload(&f->band, band) &&
                     upload(&f->twy, roots(by.L)) && upload(&f->twx, roots(bx.L)) &&
                     try_alloc(&f->w0, ws) && try_alloc(&f->w1, ws) &&

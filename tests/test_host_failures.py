@@ -1,4 +1,5 @@
-"""Allocation failures that a caller recovers from, on the host (no GPU)."""
+"""Allocation failures that a caller recovers from, and the limits of what is
+allocated, on the host (no GPU)."""
 import pytest
 
 import fakecuda
@@ -104,5 +105,21 @@ def test_former_precision_serves_on_after_a_failed_selection(fake):
         n = fake.fake_launches(b"tc_conv_kernel")
         assert h.forward() == 0 and h.adjoint() == 0, fake.swopt_last_error()
         assert fake.fake_launches(b"tc_conv_kernel") == n + 2
+    finally:
+        h.close()
+
+
+@pytest.mark.parametrize("P,N,served", [(1, 1, True), (8, 1, False), (1, 8, False)])
+def test_workspaces_stay_within_their_limit(fake, P, N, served):
+    """8 GB per workspace, whether the planes are states or species; a scan that
+    needs more is served by the direct kernels."""
+    fake.fake_largest()
+    h = fakecuda.Handle(fake, X=700, Y=700, Z=512, T=4, N=N, P=P, k=1, cycle=N)
+    try:
+        # the rest of a handle: state images, N (or P) 700^2 512 floats
+        assert fake.fake_largest() <= 8e9 + 0.1e9
+        n = fake.fake_launches(b"spec_kernel")
+        assert h.forward() == 0
+        assert (fake.fake_launches(b"spec_kernel") > n) == served
     finally:
         h.close()
