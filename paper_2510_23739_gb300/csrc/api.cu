@@ -429,7 +429,7 @@ swopt_status refined_gradient(swopt_handle* h, const float* v, const float* ytil
     const float alpha = (float)h->step;
     if (route_fft(h)) {
         FftImage img;
-        img.mode = 2;
+        img.refine = true;
         img.add = add;
         img.alpha = alpha;
         img.out = h->zin;
@@ -662,7 +662,7 @@ swopt_status fista_iteration(swopt_handle* h, int kind, cudaStream_t st)
         }
         if (one_chain && (rounds(h) || !round2)) {
             FftImage img;
-            img.mode = 2;
+            img.refine = true;
             img.alpha = alpha;
             img.out = h->zin;
             img.xi = h->xi;

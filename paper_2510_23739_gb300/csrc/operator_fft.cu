@@ -706,7 +706,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_y_kernel(const YPass a)
         });
 }
 
-enum { IMG_STORE = 0, IMG_STEP = 1, IMG_REFINE = 2 };
+enum { IMG_STORE = 0, IMG_REFINE = 1 };
 
 struct XInverse {
     FftShape s;
@@ -720,7 +720,7 @@ struct XInverse {
     const float* ytil;
     const float* Cmf;   // null: no scale
     const float* c;     // input of A (terms of its marked positions)
-    // images: IMG_STORE out = v; IMG_STEP out = xi - alpha v; IMG_REFINE as pt_refine_kernel
+    // images: IMG_STORE out = v; IMG_REFINE as pt_refine_kernel
     int add, add2;
     float alpha;
     const float* xi;
@@ -841,7 +841,7 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
                     const int gx = b + i < R ? out_x(b + i) : -1;
                     go[i] = xi[i] = make_float2(0.f, 0.f);
                     if (MODE == IMG_REFINE && gx >= 0) go[i] = get(a.G + at(gx));
-                    if (MODE != IMG_STORE && gx >= 0) xi[i] = get(a.xi + at(gx));
+                    if (MODE == IMG_REFINE && gx >= 0) xi[i] = get(a.xi + at(gx));
                 }
 #pragma unroll
                 for (int i = 0; i < CH; ++i) {
@@ -853,10 +853,9 @@ __global__ void __launch_bounds__(kMaxFftThreads, 3) fft_x_image_kernel(const XI
                         put(a.G + at(gx), g);
                         g = make_float2(fmaf(beta, g.x - go[i].x, g.x),
                                         fmaf(beta, g.y - go[i].y, g.y));
-                    }
-                    if (MODE != IMG_STORE)
                         g = make_float2(fmaf(-a.alpha, g.x, xi[i].x),
                                         fmaf(-a.alpha, g.y, xi[i].y));
+                    }
                     put(a.out + at(gx), g);
                 }
             }
@@ -944,7 +943,8 @@ struct XResidual {
 
 constexpr double kHugeYsq = 7.9228162514264338e28;  // 2^96
 
-// 112 registers: three blocks of 6 warps per SM, without spills
+// 96 registers, three blocks of 6 warps per SM (at 80 the spills cost more than the
+// fourth block gave); 48 bytes are spilled.
 __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual a)
 {
     extern __shared__ float2 sm[];
@@ -1933,10 +1933,8 @@ swopt_status adjoint_from_lines(swopt_handle* h, const FftShape& s, const float*
     v.per_state = img.per_state ? 1 : 0;
     v.vec = (h->Z % 2) == 0 && aligned8(img.out) && aligned8(img.xi) && aligned8(img.G);
     return launch_lines(h,
-                        img.mode == IMG_STORE  ? fft_x_image_kernel<IMG_STORE>
-                        : img.mode == IMG_STEP ? fft_x_image_kernel<IMG_STEP>
-                                               : fft_x_image_kernel<IMG_REFINE>,
-                        v, v.items, f->x, st);
+                        img.refine ? fft_x_image_kernel<IMG_REFINE> : fft_x_image_kernel<IMG_STORE>, v,
+                        v.items, f->x, st);
 }
 
 }  // namespace

@@ -367,12 +367,12 @@ swopt_status fft_weights(swopt_handle* h);
 // h->u = (scale ? Cm : 1) A P c - ytil (ytil may be null)
 swopt_status fft_forward(swopt_handle* h, const float* c, const float* ytil, int scale, bool round,
                          cudaStream_t st);
-// What the last kernel of A^T writes: per_state, the images g [Q][Y][X][Z]
-// (mode 0); else with v = P^T A^T, mode 0 out = v, 1 out = xi - alpha v,
-// 2 as launch_pt_refine.
+// What the last kernel of A^T writes: per_state, the images g [Q][Y][X][Z]; else
+// out = v with v = P^T A^T, or (refine) G and out as launch_pt_refine.
 struct FftImage {
     bool per_state = false;
-    int mode = 0, add = 0, add2 = 0;
+    bool refine = false;
+    int add = 0, add2 = 0;
     float alpha = 0.f;
     float* out = nullptr;
     const float* xi = nullptr;
@@ -390,7 +390,7 @@ swopt_status fft_normal(swopt_handle* h, const float* c, const float* ytil, bool
 // The refined solve's step decided on the device, in one chain of launches: by
 // h->sched[0], 0: G += H^T H delta with operands rounded if `round`; else
 // G = H^T (H c - ytil), rounded if `round2`; the rest as launch_pt_refine
-// (img.mode 2).  Only where fft_refine_gated (one tile), and not with round2
+// (img.refine).  Only where fft_refine_gated (one tile), and not with round2
 // alone.
 bool fft_refine_gated(const swopt_handle* h);
 swopt_status fft_refine(swopt_handle* h, const float* delta, const float* c, const float* ytil,
