@@ -1096,8 +1096,10 @@ __global__ void counter_random_kernel(float* x, size_t n, uint64_t seed)
 // sums its run of positions, lanes along j; parts[chunk][m][p][j] are then
 // added in chunk order.  Products are summed as in red_dot_kernel, 16 positions
 // at a time.  One thread per (m, p, j) over all positions, as it was, left all
-// but a few warps of the chip idle: 600 us at 48 x 48 x 117, now 12 us.
-__global__ void __launch_bounds__(128) param_partial_kernel(const float* __restrict__ g,
+// but a few warps of the chip idle: 600 us at 48 x 48 x 117, now 10 us.  64 registers,
+// so that the eight blocks per SM of param_weights' plan are one wave: 74 us at
+// 3 x 128^2 x 96 with 10 states, where 72 registers took 90.
+__global__ void __launch_bounds__(128, 8) param_partial_kernel(const float* __restrict__ g,
                                                             const float* __restrict__ c,
                                                             double* __restrict__ parts, int Q,
                                                             int P, int S, int Z, int run)
