@@ -78,7 +78,17 @@ typedef struct {
  * (every precision but FP8; BF16 rounds both operands first, the split
  * precisions keep FP32 operands), else, or when a tensor-core tiling or
  * schedule is pinned (swopt_tc_configure, swopt_tc_schedule), by the kernels
- * named here.
+ * named here.  The geometry allows the FFTs where the time window has at most
+ * 1376 to 1712 samples (more depths, fewer samples), the kernel's spectrum
+ * takes up to 24 GB and a workspace up to 8 GB, and the device has that memory
+ * when the handle is created (or BF16 is selected).
+ * Error of the FFTs: 1e-7 to 2e-7 of the output's norm.  It is relative to the
+ * largest values of an image (a switching state or species, two neighbouring
+ * depths or samples), so that outputs which the direct sums leave exactly zero
+ * hold about 1e-7 of the image's largest, and small outputs beside large ones
+ * have less relative accuracy than by direct sums.  Infinities, NaNs and
+ * magnitudes from 2^64 in the input do not go through the FFTs: they reach the
+ * outputs whose sums contain them, and no others.
  *  SWOPT_PREC_FP32 : FP32 FMA on the CUDA cores (the accuracy reference).
  *  SWOPT_PREC_BF16 : tcgen05 tensor cores, BF16 operands, FP32 accumulation.
  *  SWOPT_PREC_BF16X3: tcgen05 tensor cores on a two-term BF16 split of both
@@ -196,7 +206,8 @@ swopt_status swopt_create(const swopt_geometry* geom, const double* K_host,
 /* Release a handle and all device memory it owns (NULL is a no-op). */
 swopt_status swopt_destroy(swopt_handle* h);
 
-/* Select the contraction arithmetic for later calls (swopt_precision). */
+/* Select the contraction arithmetic for later calls (swopt_precision).  On
+ * failure (UNSUPPORTED geometry, OOM) the former precision stays selected. */
 swopt_status swopt_set_precision(swopt_handle* h, int precision);
 
 /* Forward operator, y = H c = W_tot S c (Eq. full-forward): for every pulse n

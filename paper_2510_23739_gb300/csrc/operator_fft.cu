@@ -1062,10 +1062,10 @@ __global__ void __launch_bounds__(288, 2) fft_x_residual_kernel(const XResidual 
 // ring of asynchronous copies that runs ahead across the warp's groups and
 // starts before the inputs are staged; a thread reads back only what it copied
 // itself, so the ring needs no barrier.
-// Bound by latency and shared-memory reads at 14 to 16 warps per SM (the inputs
-// of 10 states take 61 KB per block): 145 us per product of the largest workload
-// (k = 31, 10 states), where the K^ stream alone is 56 us of HBM time and the FMAs
-// 48 us.  One register accumulator per value with K^ read by the thread itself:
+// Bound by latency at 12 to 14 warps per SM (the inputs of 10 states take 61 KB per
+// block): 145 us per product of the largest workload (k = 31, 10 states), where the K^
+// stream alone is 56 us of HBM time and the FMAs 48 us.  The schedulers issue in 0.46
+// to 0.55 of the cycles; the first stalls are loads in flight and the FMA pipe.  One register accumulator per value with K^ read by the thread itself:
 // 200 us (164 to 255 registers, one block per SM).
 // ---------------------------------------------------------------------------
 struct Spec {
