@@ -80,7 +80,8 @@ typedef struct {
  * schedule is pinned (swopt_tc_configure, swopt_tc_schedule), by the kernels
  * named here.  The geometry allows the FFTs where the time window has at most
  * 1376 to 1712 samples (more depths, fewer samples), the kernel's spectrum
- * takes up to 24 GB and a workspace up to 8 GB, and the device has that memory
+ * takes up to 24 GB and a workspace up to 8 GB for the states' images (P / Q of
+ * it where there are more species than states), and the device has that memory
  * when the handle is created (or BF16 is selected).
  * Error of the FFTs: 1e-7 to 2e-7 of the output's norm.  It is relative to the
  * largest values of an image (a switching state or species, two neighbouring

@@ -289,7 +289,7 @@ bool use_tc(const swopt_handle* h) { return h->precision != SWOPT_PREC_FP32; }
 // FP8, unless a tensor-core tiling or schedule is pinned (swopt_tc_configure,
 // swopt_tc_schedule), which asks for those kernels, or fft_prepare left h->fft null
 // (windows over 1376 to 1712 samples, of which the product cannot stage two states;
-// 24 GB of K^, 8 GB per workspace; a failed allocation).  No line by support or size:
+// 24 GB of K^, 8 GB of states' planes per workspace; a failed allocation).  No line by support or size:
 // one FISTA iteration without TV, us, direct kernels / spectral ones, 10 states:
 //                      k = 1         k = 3         k = 7         k = 11
 //   16^2 x 24   FP32   88 / 50      218 / 50      895 / 50     2767 / 52

@@ -1699,8 +1699,9 @@ void fft_prepare(swopt_handle* h)
             const double kbytes = 0.5 * area * (frows + arows) * kOG * 8.0;
             const double sbytes = tiles * area * 8.0 * 8.0 * (h->P * Cz2 + states * Ct2);
             const double flops = tiles * 0.5 * area * (frows + arows) * kOG * 8.0 * states;
-            const double work = 8.0 * tiles * area * (double)planes;
-            // memory limits: 24 GB of K^ (twice with the BF16 one), 8 GB per workspace
+            const double work = 8.0 * tiles * area * h->Q * (double)std::max(Ct2, Cz2);
+            // memory limits: 24 GB of K^ (twice with the BF16 one), 8 GB of a workspace for
+            // the states' planes (with more species than states it takes up to P / Q of that)
             if (kbytes > 24e9 || work > 8e9) continue;
             double t = std::max(kbytes / 5e12, flops / 40e12) + sbytes / 5e12;
             if (h->r == 0) t *= 1.0 + 0.02 * tiles;

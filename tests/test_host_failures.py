@@ -109,15 +109,16 @@ def test_former_precision_serves_on_after_a_failed_selection(fake):
         h.close()
 
 
-@pytest.mark.parametrize("P,N,served", [(1, 1, True), (8, 1, False), (1, 8, False)])
-def test_workspaces_stay_within_their_limit(fake, P, N, served):
-    """8 GB per workspace, whether the planes are states or species; a scan that
-    needs more is served by the direct kernels."""
+@pytest.mark.parametrize("P,N,served", [(1, 1, True), (8, 1, True), (1, 8, False)])
+def test_workspaces_and_their_limit(fake, P, N, served):
+    """8 GB per workspace for the states' planes, or the direct kernels serve; with
+    more species than states the depths of all species (256 pairs on 9 tiles of
+    256 x 256), and no more than that."""
     fake.fake_largest()
     h = fakecuda.Handle(fake, X=700, Y=700, Z=512, T=4, N=N, P=P, k=1, cycle=N)
     try:
-        # the rest of a handle: state images, N (or P) 700^2 512 floats
-        assert fake.fake_largest() <= 8e9 + 0.1e9
+        largest = fake.fake_largest()
+        assert largest == 8 * 9 * 256**2 * 256 * P if served else largest <= 8.1e9
         n = fake.fake_launches(b"spec_kernel")
         assert h.forward() == 0
         assert (fake.fake_launches(b"spec_kernel") > n) == served
