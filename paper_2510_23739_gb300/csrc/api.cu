@@ -331,6 +331,17 @@ swopt_status prepare_route(swopt_handle* h)
     return route_fft(h) ? SWOPT_OK : tc_prepare(h);
 }
 
+// UNSUPPORTED for a precision that the tensor-core kernels do not take on the handle's
+// geometry, also where the transforms would.
+swopt_status supported_precision(swopt_handle* h)
+{
+    const unsigned bit = 1u << h->precision;
+    if (!use_tc(h) || (h->tc_takes & bit)) return SWOPT_OK;
+    SW_TRY(tc_supported(h));
+    h->tc_takes |= bit;  // the geometry and the kernel do not change
+    return SWOPT_OK;
+}
+
 // The tensor-core operator of the selected precision, built if the spectral
 // kernels do not serve it (synchronises; never called while capturing).
 swopt_status ensure_tc(swopt_handle* h)
@@ -579,6 +590,7 @@ swopt_status ensure_ref(swopt_handle* h)
     const int rp = h->prm.refine_precision;
     if (h->prm.refine_every <= 0 || rp == SWOPT_PREC_FP32 || rp == h->precision) return SWOPT_OK;
     RefScope sc(h, rp);
+    SW_TRY(supported_precision(h));
     return prepare_route(h);
 }
 
@@ -1021,8 +1033,7 @@ swopt_status swopt_set_precision(swopt_handle* h, int precision)
         const int prev = h->precision;
         h->precision = precision;
         h->no_bf16_spectrum = false;  // another try
-        // a geometry that the tensor-core kernels refuse stays refused
-        swopt_status s = tc_supported(h);
+        swopt_status s = supported_precision(h);
         if (s == SWOPT_OK) s = prepare_route(h);
         if (s != SWOPT_OK) {
             // back to the former precision, whose operator may have made room

@@ -239,6 +239,7 @@ struct swopt_handle {
     // spectral path
     swopt::FftOperator* fft = nullptr;  // null: the direct kernels serve every precision
     bool no_bf16_spectrum = false;      // no memory for it: tensor-core kernels serve BF16
+    unsigned tc_takes = 0;              // precisions found to be supported (bits)
 
     // tensor-core path
     swopt::TcOperator* tc = nullptr;      // operator of `precision`

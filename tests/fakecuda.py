@@ -74,6 +74,10 @@ class Handle:
     def adjoint(self):
         return self.L.swopt_adjoint(self.h, self.y.ctypes.data, self.x.ctypes.data, None)
 
+    def fista_init(self, **kw):
+        prm = sw.SolveParams(**kw)._c()
+        return self.L.swopt_fista_init(self.h, self.y.ctypes.data, ctypes.byref(prm), None)
+
     def objective(self):
         F, fit = ctypes.c_double(), ctypes.c_double()
         return self.L.swopt_objective(self.h, self.c.ctypes.data, self.y.ctypes.data, 0.1, 0.1, 0.0,

@@ -1,10 +1,10 @@
 """Allocation failures that a caller recovers from, and the limits of what is
-allocated, on the host (no GPU)."""
+accepted, on the host (no GPU)."""
 import pytest
 
 import fakecuda
 
-OOM, CUDA = 4, 3
+OOM, CUDA, UNSUPPORTED = 4, 3, 7
 
 
 @pytest.fixture(scope="module")
@@ -122,5 +122,23 @@ def test_workspaces_and_their_limit(fake, P, N, served):
         n = fake.fake_launches(b"spec_kernel")
         assert h.forward() == 0
         assert (fake.fake_launches(b"spec_kernel") > n) == served
+    finally:
+        h.close()
+
+
+@pytest.mark.parametrize("kw,geometry,takes", [
+    (dict(T=256), "window", True), (dict(T=257), "window", False),
+    (dict(Z=256, T=8), "depths", True), (dict(Z=257, T=8), "depths", False)])
+@pytest.mark.parametrize("resync", ["bf16", "bf16x3"])
+def test_resync_precisions_that_the_tensor_cores_refuse(fake, kw, geometry, takes, resync):
+    """A refined FP32 solve refuses a resync precision where selecting it is
+    refused, although the transforms would serve it."""
+    h = fakecuda.Handle(fake, **kw)
+    try:
+        for _ in range(2):
+            st = h.fista_init(step=0.1, lambda_tv=0.0, refine_every=2, refine_precision=resync)
+            assert st == (0 if takes else UNSUPPORTED)
+        assert h.precision(resync) == st
+        assert h.fista_init(step=0.1, lambda_tv=0.0, refine_every=2, refine_precision="fp32") == 0
     finally:
         h.close()
